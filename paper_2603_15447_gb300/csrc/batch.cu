@@ -184,31 +184,6 @@ __global__ void __launch_bounds__(256, 5) k_batch_setup(const BatchArgs a, int64
 
 // ---------------------------------------------------------------- evaluation
 
-// Grid values t_j = fl32(j) / fl32(n - 1), the IEEE quotient.  For
-// n - 1 < 2^16 without a division: q0 = RN(j r) with r = RN(1 / (n - 1)),
-// then one correction step q0 + RN(j - q0 (n - 1)) r with both steps fused
-// (Markstein's reciprocal-based division, 1990).  For every 0 <= j <= n - 1
-// < 2^16 this equals the IEEE quotient (checked exhaustively, and the exact
-// x = t of a degree-1 test curve is compared bit for bit on the GPU); larger
-// grids divide.
-struct GridDiv {
-    float den, r;
-    bool fast;
-    __device__ __forceinline__ void init(int n)
-    {
-        den = (float)(n - 1);
-        r = __frcp_rn((float)(n > 1 ? n - 1 : 1));
-        fast = n > 1 && n - 1 < 65536;
-    }
-    __device__ __forceinline__ float operator()(int j) const
-    {
-        const float fj = (float)j;
-        if (!fast) return den > 0.f ? __fdiv_rn(fj, den) : 0.f;
-        const float q0 = __fmul_rn(fj, r);
-        return fmaf(fmaf(-q0, den, fj), r, q0);
-    }
-};
-
 // Span of t given the span s of an earlier, smaller parameter of the same
 // run: the residual fma(t, ns, -s) is >= 0 with its exact sign, so s stands
 // unless it reaches 1, when the full selection runs.  Same s and tau as

@@ -74,10 +74,13 @@ __device__ __forceinline__ float lerp(float a, float b, float t)
     return fmaf(t, b, fmaf(-t, a, a));
 }
 
-// clamp to [0,1] keeping NaN (fminf/fmaxf would drop it)
+// clamp to [0,1] keeping NaN (fminf/fmaxf would drop it): two instructions,
+// where comparisons and selects take four
 __device__ __forceinline__ float clamp01(float t)
 {
-    return t < 0.f ? 0.f : (t > 1.f ? 1.f : t);
+    float r;
+    asm("max.NaN.f32 %0, %1, 0f00000000;\n\tmin.NaN.f32 %0, %0, 0f3F800000;" : "=f"(r) : "f"(t));
+    return r;
 }
 
 __device__ __forceinline__ float sqrt_approx(float x)
@@ -120,5 +123,30 @@ __device__ __forceinline__ float warp_sum16_scatter(float (&v)[16], int lane)
     }
     return v[0] + __shfl_xor_sync(kFull, v[0], 1);
 }
+
+// Grid values t_j = fl32(j) / fl32(n - 1), the IEEE quotient.  For
+// n - 1 < 2^16 without a division: q0 = RN(j r) with r = RN(1 / (n - 1)),
+// then one correction step q0 + RN(j - q0 (n - 1)) r with both steps fused
+// (Markstein's reciprocal-based division, 1990).  For every 0 <= j <= n - 1
+// < 2^16 this equals the IEEE quotient (checked exhaustively, and the exact
+// x = t of a degree-1 test curve is compared bit for bit on the GPU); larger
+// grids divide.
+struct GridDiv {
+    float den, r;
+    bool fast;
+    __device__ __forceinline__ void init(int n)
+    {
+        den = (float)(n - 1);
+        r = __frcp_rn((float)(n > 1 ? n - 1 : 1));
+        fast = n > 1 && n - 1 < 65536;
+    }
+    __device__ __forceinline__ float operator()(int j) const
+    {
+        const float fj = (float)j;
+        if (!fast) return den > 0.f ? __fdiv_rn(fj, den) : 0.f;
+        const float q0 = __fmul_rn(fj, r);
+        return fmaf(fmaf(-q0, den, fj), r, q0);
+    }
+};
 
 }  // namespace bez

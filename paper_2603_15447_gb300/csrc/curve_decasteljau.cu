@@ -1,5 +1,5 @@
-// curve_decasteljau.cu -- instantiates the decasteljau register evaluator (see curve_eval.cuh).
-#include "curve_eval.cuh"
+// curve_decasteljau.cu -- instantiates the decasteljau register evaluator (see curve_tile.cuh).
+#include "curve_tile.cuh"
 
 namespace bez {
 LaunchResult launch_curve_decasteljau(const CurveArgs& a, int tm, int om, cudaStream_t s, const LaunchHooks& h)

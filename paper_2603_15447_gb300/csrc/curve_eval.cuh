@@ -1,7 +1,9 @@
-// curve_eval.cuh -- register evaluators for Bezier curves and the kernels that
-// drive them: one curve per warp (every variant), and for the fused
-// evaluate-and-measure form of centred Horner on 3D curves of degree <= 4 two
-// curves per warp (k_curve_pair) or 8 / 4 lanes per curve (k_curve_group).
+// curve_eval.cuh -- register evaluators for Bezier curves and kernels that drive
+// them: one curve per warp (k_curve: runtime degrees, and the fused
+// draw-and-measure form of 3D curves), and for that form of centred Horner on
+// degree <= 4 two curves per warp (k_curve_pair) or 8 / 4 lanes per curve
+// (k_curve_group).  Points and other lengths of degree 1..7, any dimension:
+// curve_tile.cuh.
 //
 // Each evaluator is a struct with setup(b) (per curve, once) and eval(t, P)
 // (per parameter).  D is the degree when known at compile time, or 0 for the
@@ -424,8 +426,8 @@ struct Eval<VAR_SEILER, D, DIM> {
 
 // ---------------------------------------------------------------- runtime degree
 
-// Fallback for degrees not instantiated at compile time (and for dim != 3):
-// the same arithmetic as the fixed-degree evaluators, written with plain
+// Fallback for degrees not instantiated at compile time (8..15): the same
+// arithmetic as the fixed-degree evaluators, written with plain
 // loops over the runtime degree.  Setup is FP64 from degree 8 on.
 template <int VAR, int DIM>
 struct EvalDyn {
@@ -953,51 +955,6 @@ LaunchResult launch_one(const CurveArgs& a, cudaStream_t s, const LaunchHooks& h
     cudaError_t err = cudaGetLastError();
     h.end(h.self, s);
     return {1, err};
-}
-
-template <int VAR, int D, int DIM>
-LaunchResult launch_modes(const CurveArgs& a, int tm, int om, cudaStream_t s, const LaunchHooks& h)
-{
-    if (om == OM_POINTS) {
-        if (tm == TM_ARRAY) return launch_one<VAR, D, DIM, TM_ARRAY, OM_POINTS>(a, s, h);
-        if (tm == TM_UNIFORM) return launch_one<VAR, D, DIM, TM_UNIFORM, OM_POINTS>(a, s, h);
-        return launch_one<VAR, D, DIM, TM_HASH, OM_POINTS>(a, s, h);
-    }
-    if (tm == TM_ARRAY) return launch_one<VAR, D, DIM, TM_ARRAY, OM_LENGTH>(a, s, h);
-    if (tm == TM_UNIFORM) return launch_one<VAR, D, DIM, TM_UNIFORM, OM_LENGTH>(a, s, h);
-    // the fused evaluate-and-measure form of 3D curves of fixed degree gets the
-    // pre-mixed draw when every sample index fits 16 bits; centred Horner up
-    // to degree 4 runs two curves per warp from 64 samples, four from 128 and
-    // eight from 256
-    if constexpr (VAR == VAR_HORNER_CENTRED && D > 0 && D <= 4 && DIM == 3) {
-        if (a.n_t >= kGroup4MinSamples && a.n_t <= 65536) return launch_group<D, 4>(a, s, h);
-        if (a.n_t >= kGroup8MinSamples && a.n_t <= 65536) return launch_group<D, 8>(a, s, h);
-        if (a.n_t >= 64 && a.n_t <= 65536) return launch_pair<D>(a, s, h);
-    }
-    if (D > 0 && DIM == 3 && a.n_t <= 65536) return launch_one<VAR, D, DIM, (D > 0 && DIM == 3 ? TM_HASH16 : TM_HASH), OM_LENGTH>(a, s, h);
-    return launch_one<VAR, D, DIM, TM_HASH, OM_LENGTH>(a, s, h);
-}
-
-template <int VAR>
-LaunchResult launch_curve_variant(const CurveArgs& a, int tm, int om, cudaStream_t s, const LaunchHooks& h)
-{
-    if (a.dim == 3) {
-        switch (a.degree) {
-        case 1: return launch_modes<VAR, 1, 3>(a, tm, om, s, h);
-        case 2: return launch_modes<VAR, 2, 3>(a, tm, om, s, h);
-        case 3: return launch_modes<VAR, 3, 3>(a, tm, om, s, h);
-        case 4: return launch_modes<VAR, 4, 3>(a, tm, om, s, h);
-        case 5: return launch_modes<VAR, 5, 3>(a, tm, om, s, h);
-        case 6: return launch_modes<VAR, 6, 3>(a, tm, om, s, h);
-        case 7: return launch_modes<VAR, 7, 3>(a, tm, om, s, h);
-        default: return launch_modes<VAR, 0, 3>(a, tm, om, s, h);
-        }
-    }
-    switch (a.dim) {
-    case 1: return launch_modes<VAR, 0, 1>(a, tm, om, s, h);
-    case 2: return launch_modes<VAR, 0, 2>(a, tm, om, s, h);
-    default: return launch_modes<VAR, 0, 4>(a, tm, om, s, h);
-    }
 }
 
 }  // namespace bez
