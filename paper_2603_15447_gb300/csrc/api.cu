@@ -665,17 +665,22 @@ static bez_status eval_spline(bez_ctx c, const float* ctrl, const float* weights
     a.err_word = o->err_word;
     const uint32_t seed_lo = (uint32_t)(o->seed & 0xffffffffu), seed_hi = (uint32_t)(o->seed >> 32);
     a.key = lowbias32(seed_lo ^ lowbias32(seed_hi ^ lowbias32(o->stream_id)));
-    // Bezier spans: library-owned scratch, one slot per context
-    const size_t span_bytes = (size_t)n_curves * a.n_spans * (degree + 1) * a.comps * sizeof(float);
-    st = ensure_stage(c, 5, span_bytes, s);
-    if (st != BEZ_OK) return st;
-    a.spans = static_cast<float*>(c->stage[5].p);
     const int tm = t_array ? TM_ARRAY : (o->t_mode == BEZ_T_UNIFORM ? TM_UNIFORM : TM_HASH);
     const int om = o->out_mode == BEZ_OUT_POINTS ? OM_POINTS : OM_LENGTH;
     LaunchHooks h = hooks_of(c);
-    LaunchResult r = launch_spline_setup(a, s, h);
-    if (r.err != cudaSuccess) return cuda_fail(r.err, "spline setup launch");
-    r = launch_spline_eval(a, tm, om, s, h);
+    LaunchResult r{0, cudaSuccess};
+    if (spline_fits_fused(a)) {
+        r = launch_spline_fused(a, tm, om, s, h);
+    } else {
+        // Bezier spans: library-owned scratch, one slot per context
+        const size_t span_bytes = (size_t)n_curves * a.n_spans * (degree + 1) * a.comps * sizeof(float);
+        st = ensure_stage(c, 5, span_bytes, s);
+        if (st != BEZ_OK) return st;
+        a.spans = static_cast<float*>(c->stage[5].p);
+        r = launch_spline_setup(a, s, h);
+        if (r.err != cudaSuccess) return cuda_fail(r.err, "spline setup launch");
+        r = launch_spline_eval(a, tm, om, s, h);
+    }
     if (r.err != cudaSuccess) return cuda_fail(r.err, "spline evaluator launch");
     return stg.finish(o->sync);
 }

@@ -136,6 +136,10 @@ struct SplineArgs {
 };
 LaunchResult launch_spline_setup(const SplineArgs& a, cudaStream_t s, const LaunchHooks& h);
 LaunchResult launch_spline_eval(const SplineArgs& a, int tm, int om, cudaStream_t s, const LaunchHooks& h);
+// Extraction and evaluation in one kernel, for splines that fit it (degree
+// 1..5, a curve's spans in shared memory); needs no span scratch.
+bool spline_fits_fused(const SplineArgs& a);
+LaunchResult launch_spline_fused(const SplineArgs& a, int tm, int om, cudaStream_t s, const LaunchHooks& h);
 
 // ---------------------------------------------------------------- surfaces / volumes
 

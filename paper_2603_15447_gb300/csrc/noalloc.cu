@@ -156,8 +156,13 @@ extern "C" bez_status bez_eval_spline_noalloc(const float* ctrl, const float* we
     const int om = o->out_mode == BEZ_OUT_POINTS ? OM_POINTS : OM_LENGTH;
     const LaunchHooks h{no_count, no_event, no_event, nullptr, sm_count};
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    LaunchResult r = launch_spline_setup(a, s, h);
-    if (r.err == cudaSuccess) r = launch_spline_eval(a, tm, om, s, h);
+    LaunchResult r{0, cudaSuccess};
+    if (spline_fits_fused(a)) {
+        r = launch_spline_fused(a, tm, om, s, h);
+    } else {
+        r = launch_spline_setup(a, s, h);
+        if (r.err == cudaSuccess) r = launch_spline_eval(a, tm, om, s, h);
+    }
     if (r.err != cudaSuccess) return fail_na(BEZ_ERR_CUDA, cudaGetErrorString(r.err));
     if (o->sync) {
         e = cudaStreamSynchronize(s);

@@ -1,6 +1,8 @@
 // spline.cu -- B-spline and NURBS evaluation (paper Sec. 2.2): FP64 Boehm
 // extraction of every span's Bezier control points, then FP32 de Casteljau
 // on the span that holds each parameter.  See spline.cuh for the algorithm.
+// Splines of degree 1..5 whose spans fit in shared memory take one fused kernel
+// instead (spline_fused.cuh).
 #include "curve_eval.cuh"
 #include "spline.cuh"
 
