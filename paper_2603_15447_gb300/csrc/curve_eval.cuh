@@ -93,6 +93,22 @@ constexpr CentredTables make_centred_tables()
 }
 static __constant__ CentredTables kCentredT = make_centred_tables();
 
+// T_d of one degree in FP32 (exact), small enough for the compiler to turn
+// constant-index reads into immediate operands.
+template <int D>
+struct CentredMatrix {
+    float t[D + 1][D + 1];
+};
+template <int D>
+constexpr CentredMatrix<D> make_centred_matrix()
+{
+    CentredMatrix<D> r{};
+    const CentredTables all = make_centred_tables();
+    for (int m = 0; m <= D; ++m)
+        for (int i = 0; i <= D; ++i) r.t[m][i] = (float)all.t[D][m][i];
+    return r;
+}
+
 // ---------------------------------------------------------------- evaluators
 
 template <int VAR, int D, int DIM>
