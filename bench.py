@@ -65,7 +65,7 @@ T_OPS, LEN_OPS = 9, 8
 # on the full 65,536 x 512 fit step.
 TRAFFIC_PER_CURVE = {"HORNER_CENTRED": 6312448 / 131072}
 # the kernel behind each headline variant's fused length (cubic 3D, hashed t)
-KERNEL_NAME = {"HORNER_CENTRED": "k_curve_group<3, 4> (four lanes per curve)", "HALF2": "k_curve_h2"}
+KERNEL_NAME = {"HORNER_CENTRED": "k_length<2, 3, 3, true> (four lanes per curve, two samples per instruction)", "HALF2": "k_curve_h2"}
 TRAFFIC_SURFACE_65536 = 12652544 + 742988544
 TRAFFIC_FIT_65536x512 = 540180736 + 121996800
 EVAL_OPS = {"HORNER": 9, "HORNER_CENTRED": 9, "HALF2": 5, "BERNSTEIN": 19, "SEILER": 16, "DECASTELJAU": 36,

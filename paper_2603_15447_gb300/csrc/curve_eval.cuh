@@ -1,9 +1,7 @@
 // curve_eval.cuh -- register evaluators for Bezier curves and kernels that drive
 // them: one curve per warp (k_curve: runtime degrees, and the fused
-// draw-and-measure form of 3D curves), and for that form of centred Horner on
-// degree <= 4 two curves per warp (k_curve_pair) or 8 / 4 lanes per curve
-// (k_curve_group).  Points and other lengths of degree 1..7, any dimension:
-// curve_tile.cuh.
+// draw-and-measure form of 3D curves except for centred Horner).  Points and
+// other lengths of degree 1..7, any dimension: curve_tile.cuh.
 //
 // Each evaluator is a struct with setup(b) (per curve, once) and eval(t, P)
 // (per parameter).  D is the degree when known at compile time, or 0 for the
@@ -91,7 +89,6 @@ constexpr CentredTables make_centred_tables()
         }
     return r;
 }
-static __constant__ CentredTables kCentredT = make_centred_tables();
 
 // T_d of one degree in FP32 (exact), small enough for the compiler to turn
 // constant-index reads into immediate operands.
@@ -195,63 +192,6 @@ struct Eval<VAR_HORNER_CENTRED, D, DIM> {
         d = Deg<D>::get(deg);
         if (d >= kFp64SetupCentred) setup_t<double>(b);
         else setup_t<float>(b);
-    }
-    // Warp-cooperative setup for 3D curves of fixed degree: the curve's
-    // control points are spread one element per lane (lane 3i + k holds
-    // b_i[k], in v); lane 3m + k forms a[m][k] = sum_i T_d[m][i] b_i[k] (FP64
-    // from degree 5, like setup) and the warp broadcasts the coefficients.
-    // One dot product per lane instead of the whole conversion per lane.
-    // base: first lane of the group holding the curve (0 for a whole warp;
-    // 0 or 16 when two curves share a warp)
-    __device__ __forceinline__ void setup_warp(float v, int lane, int base = 0)
-    {
-        static_assert(D > 0 && DIM == 3 && 3 * (D + 1) <= 32, "fixed-degree 3D curves only");
-        d = D;
-        using S = typename std::conditional<(D >= kFp64SetupCentred), double, float>::type;
-        const int li = lane - base;
-        const int m = li < 3 * (D + 1) ? li / 3 : 0;
-        const int k = li < 3 * (D + 1) ? li - 3 * m : 0;
-        S acc = (S)0;
-#pragma unroll
-        for (int i = 0; i <= D; ++i) {
-            const float bik = __shfl_sync(kFull, v, base + 3 * i + k);
-            acc = fma((S)kCentredT.t[D][m][i], (S)bik, acc);
-        }
-        const float cm = (float)acc;
-#pragma unroll
-        for (int mm = 0; mm <= D; ++mm)
-#pragma unroll
-            for (int kk = 0; kk < 3; ++kk) a[mm][kk] = __shfl_sync(kFull, cm, base + 3 * mm + kk);
-    }
-    // Setup for 3D curves of fixed degree held by a group of G lanes (lane
-    // base + r, slot s of v holds element G s + r of the curve, b_i[k] being
-    // element 3 i + k): every lane gathers the 3 (D + 1) elements and forms
-    // all coefficients itself.  The operator entries are then the same for
-    // every lane (uniform constant reads), and the sums run in setup_warp's
-    // order, so the coefficients are the same as setup_warp's.
-    template <int G, int NL>
-    __device__ __forceinline__ void setup_group(const float (&v)[NL], int base)
-    {
-        static_assert(D > 0 && DIM == 3 && 3 * (D + 1) <= G * NL, "fixed-degree 3D curves only");
-        d = D;
-        using S = typename std::conditional<(D >= kFp64SetupCentred), double, float>::type;
-        float b[D + 1][3];
-#pragma unroll
-        for (int i = 0; i <= D; ++i)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const int e = 3 * i + k;
-                b[i][k] = __shfl_sync(kFull, v[e / G], base + e % G);
-            }
-#pragma unroll
-        for (int m = 0; m <= D; ++m)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                S acc = (S)0;
-#pragma unroll
-                for (int i = 0; i <= D; ++i) acc = fma((S)kCentredT.t[D][m][i], (S)b[i][k], acc);
-                a[m][k] = (float)acc;
-            }
     }
     __device__ __forceinline__ void eval(float t, float (&P)[DIM]) const { eval_u(t - 0.5f, P); }
     // evaluate at u = t - 1/2
@@ -560,11 +500,6 @@ struct Pick<VAR, 0, DIM> {
 
 constexpr int kWarps = 8;  // warps per block; one curve per warp per iteration
 constexpr int kCurvesPerWarp = 8;  // curves per warp when the grid is not persistent
-constexpr int kPairsPerWarp = 4;   // the same for the two-curves-per-warp kernel
-constexpr int kGroupUnitsPerWarp = 2;  // and for the G-lanes-per-curve kernel
-constexpr int kGroupWarps = 16;        // warps per block of the G-lanes-per-curve kernel (2 blocks per SM)
-constexpr int kGroup8MinSamples = 128;  // samples per curve from which 8 lanes take a curve
-constexpr int kGroup4MinSamples = 256;  // and from which 4 lanes do
 
 template <int TM>
 __device__ __forceinline__ float param(const CurveArgs& a, int64_t c, int j, uint32_t kc)
@@ -728,15 +663,10 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_curve(const CurveArgs a)
     cur.load(a, c, per, lane);
     for (; c < a.n_curves; c += n_warps) {
         E e;
-        if constexpr (VAR == VAR_HORNER_CENTRED && D > 0 && DIM == 3) {
-            e.setup_warp(cur.v[0], lane);
-            cur.load(a, c + n_warps, per, lane);   // prefetch the next curve of this warp
-        } else {
-            float b[N][DIM];
-            cur.unpack(b, deg);
-            cur.load(a, c + n_warps, per, lane);
-            e.setup(b, deg);
-        }
+        float b[N][DIM];
+        cur.unpack(b, deg);
+        cur.load(a, c + n_warps, per, lane);  // prefetch the next curve of this warp
+        e.setup(b, deg);
         const uint32_t kc = curve_key<TM>(a, c);
         const int n_t = a.n_t;
 
@@ -796,159 +726,7 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_curve(const CurveArgs a)
     }
 }
 
-// Two curves per warp for the fused centred-Horner length of 3D curves of
-// degree <= 4 under the pre-mixed draw: lanes 0-15 take curve 2 p, lanes
-// 16-31 curve 2 p + 1.  Each half loads its 3 (d + 1) control values with
-// one request, converts them cooperatively (setup_warp with a base lane),
-// walks runs of a multiple of 4 samples per lane and reduces its length over
-// 16 lanes, so the per-curve work (load, conversion, shuffles, reduction)
-// is shared by twice the samples of a lane compared with one curve per warp.
-// The sums run over 16 runs of about n_t / 16 samples.
-template <int D>
-__global__ void __launch_bounds__(kWarps * 32, 5) k_curve_pair(const CurveArgs a)
-{
-    using E = Eval<VAR_HORNER_CENTRED, D, 3>;
-    constexpr int PER = 3 * (D + 1);
-    static_assert(PER <= 16, "a half warp holds one curve's control values");
-    const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
-    const int half = lane >> 4, li = lane & 15, base = lane & 16;
-    const int64_t n_pairs = (a.n_curves + 1) / 2;
-    const int64_t n_warps = (int64_t)gridDim.x * kWarps;
-    auto load = [&](int64_t pr) {
-        const int64_t c = 2 * pr + half;
-        return (c < a.n_curves && li < PER) ? load_elem(a.ctrl, a.dtype, c * PER + li) : 0.f;
-    };
-    const int n_t = a.n_t;
-    const int chunk = ((n_t + 15) / 16 + 3) & ~3;
-    int64_t pr = (int64_t)blockIdx.x * kWarps + wib;
-    float v = load(pr);
-    for (; pr < n_pairs; pr += n_warps) {
-        const int64_t c = 2 * pr + half;
-        const bool live = c < a.n_curves;  // the last pair may have one curve
-        E e;
-        e.setup_warp(v, lane, base);
-        v = load(pr + n_warps);  // prefetch this warp's next pair
-        const uint32_t kc = curve_key<TM_HASH16>(a, c);
-        const int jb = li * chunk;
-        const int je = live ? min(jb + chunk, n_t) : jb;
-        float acc = 0.f;
-        float first[3] = {0.f, 0.f, 0.f}, prev[3] = {0.f, 0.f, 0.f};
-        if (jb < je) acc = run_length_h16<E, 3>(e, kc, jb, je, first, prev);
-        float pl[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) pl[k] = __shfl_up_sync(kFull, prev[k], 1);
-        if (li > 0 && jb < je) acc += seg_len<3>(first, pl);
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);  // within the half
-        if (li == 0 && live) a.out[c] = acc;
-    }
-}
-
-// G = 8 or 4 lanes per curve (4 or 8 curves per warp), for the same workload
-// with more samples per curve: lanes G g .. G g + G - 1 take curve
-// (32 / G) q + g.  Each group loads its 3 (d + 1) control values
-// (ceil(3 (d + 1) / G) per lane), converts them redundantly (setup_group),
-// walks runs of a multiple of 4 samples per lane and reduces its length over
-// G lanes.  Against two curves per warp, a lane's per-curve work (load,
-// conversion, key, run ends, reduction, store) is spread over 16 / G times
-// the samples.  The sums run over G runs of about n_t / G samples.  (One or
-// two lanes per curve measured slower at 1024 samples: 1.10e12 and 1.17e12
-// against 1.18e12 points/s for 4.)  64 registers (4 blocks per SM) with the
-// group loop unrolled by 4: 1.21e12 against 1.18e12 at 48 registers with 2;
-// 80 registers measured slower.  Blocks of 16 warps (2 per SM) measured 1 %
-// faster than 8 (4 per SM) or 4 (8 per SM).
-template <int D, int G>
-__global__ void __launch_bounds__(kGroupWarps * 32, 2) k_curve_group(const CurveArgs a)
-{
-    using E = Eval<VAR_HORNER_CENTRED, D, 3>;
-    constexpr int PER = 3 * (D + 1);
-    constexpr int NL = (PER + G - 1) / G;
-    constexpr int CPW = 32 / G;  // curves per warp
-    static_assert(G == 4 || G == 8, "4 or 8 lanes per curve");
-    const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
-    const int grp = lane / G, li = lane % G, base = lane - li;
-    const int64_t n_units = (a.n_curves + CPW - 1) / CPW;
-    const int64_t n_warps = (int64_t)gridDim.x * kGroupWarps;
-    float v[NL];
-    auto load = [&](int64_t q) {
-        const int64_t c = CPW * q + grp;
-#pragma unroll
-        for (int r = 0; r < NL; ++r) {
-            const int i = li + G * r;
-            v[r] = (c < a.n_curves && i < PER) ? load_elem(a.ctrl, a.dtype, c * PER + i) : 0.f;
-        }
-    };
-    const int n_t = a.n_t;
-    const int chunk = ((n_t + G - 1) / G + 3) & ~3;
-    int64_t q = (int64_t)blockIdx.x * kGroupWarps + wib;
-    load(q);
-    for (; q < n_units; q += n_warps) {
-        const int64_t c = CPW * q + grp;
-        const bool live = c < a.n_curves;  // the warp's last unit may be partial
-        E e;
-        e.template setup_group<G>(v, base);
-        load(q + n_warps);  // prefetch this warp's next curves
-        const uint32_t kc = curve_key<TM_HASH16>(a, c);
-        const int jb = li * chunk;
-        const int je = live ? min(jb + chunk, n_t) : jb;
-        float acc = 0.f;
-        float first[3] = {0.f, 0.f, 0.f}, prev[3] = {0.f, 0.f, 0.f};
-        if (jb < je) acc = run_length_h16<E, 3, 4>(e, kc, jb, je, first, prev);
-        float pl[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) pl[k] = __shfl_up_sync(kFull, prev[k], 1);
-        if (li > 0 && jb < je) acc += seg_len<3>(first, pl);
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);  // within the group
-        if (li == 0 && live) a.out[c] = acc;
-    }
-}
-
 // ---------------------------------------------------------------- dispatch
-
-// Grid of the pair kernel: as launch_one, with pairs of curves as the unit.
-template <int D>
-LaunchResult launch_pair(const CurveArgs& a, cudaStream_t s, const LaunchHooks& h)
-{
-    auto kern = k_curve_pair<D>;
-    const int64_t n_pairs = (a.n_curves + 1) / 2;
-    const int64_t work = (n_pairs + kWarps - 1) / kWarps;
-    int grid = persistent_grid((const void*)kern, kWarps * 32, 0, h.sm_count, work);
-    if (work > grid) {
-        const int64_t g = (n_pairs + (int64_t)kWarps * kPairsPerWarp - 1) / ((int64_t)kWarps * kPairsPerWarp);
-        if (g > grid) grid = (int)(g < 2147483647 ? g : 2147483647);
-    }
-    h.count(h.self);
-    h.begin(h.self, s);
-    kern<<<grid, kWarps * 32, 0, s>>>(a);
-    cudaError_t err = cudaGetLastError();
-    h.end(h.self, s);
-    return {1, err};
-}
-
-// Grid of the G-lanes-per-curve kernel: units of 32 / G curves,
-// kGroupUnitsPerWarp per warp when they outnumber the resident warps.
-template <int D, int G>
-LaunchResult launch_group(const CurveArgs& a, cudaStream_t s, const LaunchHooks& h)
-{
-    auto kern = k_curve_group<D, G>;
-    const int64_t n_units = (a.n_curves + 32 / G - 1) / (32 / G);
-    const int64_t work = (n_units + kGroupWarps - 1) / kGroupWarps;
-    int grid = persistent_grid((const void*)kern, kGroupWarps * 32, 0, h.sm_count, work);
-    if (work > grid) {
-        const int64_t per = (int64_t)kGroupWarps * kGroupUnitsPerWarp;
-        const int64_t g = (n_units + per - 1) / per;
-        if (g > grid) grid = (int)(g < 2147483647 ? g : 2147483647);
-    }
-    h.count(h.self);
-    h.begin(h.self, s);
-    kern<<<grid, kGroupWarps * 32, 0, s>>>(a);
-    cudaError_t err = cudaGetLastError();
-    h.end(h.self, s);
-    return {1, err};
-}
 
 template <int VAR, int D, int DIM, int TM, int OM>
 LaunchResult launch_one(const CurveArgs& a, cudaStream_t s, const LaunchHooks& h)

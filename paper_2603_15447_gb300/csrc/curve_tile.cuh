@@ -1,6 +1,7 @@
 // curve_tile.cuh -- the general register kernels for single curves of fixed
 // degree (1..7) and any dimension: points (k_points) and polyline lengths
-// (k_length), several curves per warp.
+// (k_length), several curves per warp, and the fused draw-and-measure form of
+// centred Horner in packed FP32 pairs.
 //
 // The parameter kind (array, uniform grid, draw) is a launch argument: a lane
 // fetches the parameters of four samples behind one uniform branch, so one
@@ -237,12 +238,180 @@ __global__ void __launch_bounds__(kWarps * 32, (D + 1) * DIM > 20 ? 3 : (D + 1) 
     }
 }
 
+// ---------------------------------------------------------------- packed lengths
+
+// Two FP32 values per register pair.  sm_103a runs add, multiply and fma on both
+// halves with one instruction of two cycles: as many operations per cycle as the
+// scalar forms, for half of the issue slots, and the fused draw-and-measure loop
+// is bound by instruction issue: 28 -> 21.5 lane instructions per point of a 3D
+// cubic.  1,048,576 cubics x 1024 draws: 868 -> 823 us (the FMA pipe that also
+// takes the integer multiplies then 76 % busy, issue 70 %; scalar subtractions,
+// additions or square-root sums, 2 or 4 samples side by side and 80 registers
+// all measured slower or the same); 65,536 x 400 of degree 5 68 -> 38 us, 2D
+// cubics 217 -> 25 us.
+using f32x2 = unsigned long long;
+
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Centred Horner at two parameters at once, u = t - 1/2.
+template <int D, int DIM>
+struct PackedHorner {
+    f32x2 c[D + 1][DIM];
+    __device__ __forceinline__ void setup(const Eval<VAR_HORNER_CENTRED, D, DIM>& e)
+    {
+#pragma unroll
+        for (int i = 0; i <= D; ++i)
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) c[i][k] = pack2(e.a[i][k], e.a[i][k]);
+    }
+    __device__ __forceinline__ void eval(f32x2 u, f32x2 (&P)[DIM]) const
+    {
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) {
+            f32x2 acc = c[D][k];
+#pragma unroll
+            for (int i = D - 1; i >= 0; --i) acc = fma2(acc, u, c[i][k]);
+            P[k] = acc;
+        }
+    }
+};
+
+// u = t - 1/2 at the pre-mixed draws of samples ja + i and jb + i, i < 4 (ja, jb
+// multiples of 4, so a draw's input is one xor from the group's).  1.m - 3/2
+// equals (1.m - 1) - 1/2, both subtractions of the scalar form being exact.
+__device__ __forceinline__ void packed_draws(uint32_t key, uint32_t ja, uint32_t jb, f32x2 (&u)[4])
+{
+    const uint32_t ka = key ^ ja, kb = key ^ jb;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        u[i] = add2(pack2(hash_one_plus(lowbias32_tail((ka ^ (uint32_t)i) * kLowbiasMul1)),
+                          hash_one_plus(lowbias32_tail((kb ^ (uint32_t)i) * kLowbiasMul1))),
+                    pack2(-1.5f, -1.5f));
+}
+
+// Length over one lane's samples [s, e): the half runs [s, m) and [m, e) side by
+// side in the halves of the packed registers, their ends joined.  s and m are
+// multiples of 4 and the halves' groups of 4 differ by at most one, so at most
+// 7 samples of the first and 3 of the second half are left for scalar steps.
+// `first`, `last`: the run's end points.
+template <int D, int DIM>
+__device__ __forceinline__ float packed_run(const Eval<VAR_HORNER_CENTRED, D, DIM>& e, const TileParams& tp,
+                                            uint32_t s, uint32_t m, uint32_t end, float (&first)[DIM],
+                                            float (&last)[DIM])
+{
+    PackedHorner<D, DIM> h;
+    h.setup(e);
+    const uint32_t both = min(m - s, end - m) & ~3u;
+    f32x2 acc2 = 0ull, prev[DIM];
+    float acc = 0.f, fb[DIM], pa[DIM], pb[DIM];
+    if (both > 0) {
+        f32x2 u[4];
+        packed_draws(tp.key, s, m, u);
+        h.eval(u[0], prev);  // the run's first segment ends where it starts: length 0
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) unpack2(prev[k], first[k], fb[k]);
+        for (uint32_t i = 0; i < both; i += 4) {
+            if (i > 0) packed_draws(tp.key, s + i, m + i, u);
+            f32x2 gs = 0ull;  // a group's 4 segments are summed first
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                f32x2 P[DIM], q = 0ull;
+                h.eval(u[g], P);
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) {
+                    const f32x2 d = sub2(P[k], prev[k]);
+                    q = k == 0 ? mul2(d, d) : fma2(d, d, q);
+                    prev[k] = P[k];
+                }
+                float qa, qb;
+                unpack2(q, qa, qb);
+                const f32x2 sl = pack2(sqrt_approx(qa), sqrt_approx(qb));
+                gs = g == 0 ? sl : add2(gs, sl);
+            }
+            acc2 = add2(acc2, gs);
+        }
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) unpack2(prev[k], pa[k], pb[k]);
+        float aa, ab;
+        unpack2(acc2, aa, ab);
+        acc = aa + ab;
+    }
+    // what is left of either half
+    auto step = [&](uint32_t j, bool start, float (&f)[DIM], float (&p)[DIM]) {
+        float t[1], P[DIM];
+        tp.get<1, true>(TM_HASH16, j, 1, 0, t);
+        e.eval(t[0], P);
+        if (start) {
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) f[k] = P[k];
+        } else {
+            acc += seg_len<DIM>(P, p);
+        }
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) p[k] = P[k];
+    };
+#pragma unroll 1
+    for (uint32_t j = s + both; j < m; ++j) step(j, j == s, first, pa);
+#pragma unroll 1
+    for (uint32_t j = m + both; j < end; ++j) step(j, j == m, fb, pb);
+    if (end > m) {
+        acc += seg_len<DIM>(fb, pa);
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) last[k] = pb[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) last[k] = pa[k];
+    }
+    return acc;
+}
+
+// resident blocks per SM that k_length's registers are sized for (the packed
+// form holds its coefficients twice)
+__host__ __device__ constexpr int length_blocks(bool packed, int D, int DIM)
+{
+    const int per = (D + 1) * DIM;
+    return packed ? (per <= 6 ? 5 : per <= 12 ? 4 : per <= 16 ? 3 : 2) : per > 20 ? 3 : 4;
+}
+
 // Polyline lengths, 2^lg lanes a curve (65,536 cubics x 400 samples: shared t
-// 36 us, uniform 35, own t 43, against 42, 48 and 52 with a warp per curve; 2D
-// draws 34 against 216 with the runtime-degree kernel): each lane walks a contiguous run of
-// samples, the segments joining two runs are closed with one shuffle, and the
+// 36 us, uniform 35, own t 43, against 42, 48 and 52 with a warp per curve): each
+// lane walks a contiguous run of samples (PACKED: centred Horner at pre-mixed
+// draws, two half runs at a time), the segments joining two runs are closed with one shuffle, and the
 // run sums are added over the curve's lanes.
-template <int VAR, int D, int DIM>
+template <int VAR, int D, int DIM, bool PACKED>
 __global__ void __launch_bounds__(kWarps * 32, (D + 1) * DIM > 20 ? 3 : (D + 1) * DIM > 12 ? 4 : 4)
     k_length(const CurveArgs a, int tm, int lg)
 {
@@ -264,43 +433,55 @@ __global__ void __launch_bounds__(kWarps * 32, (D + 1) * DIM > 20 ? 3 : (D + 1) 
         tile_setup<VAR>(a, sm, c0, nc, grp, lane, e);
         const bool live = grp < nc;
         tp.curve(a, tm, c0 + (live ? grp : 0));
-        const uint32_t jb = min(li * run, n_t), je = live ? min(jb + run, n_t) : jb;
         float acc = 0.f, first[DIM], prev[DIM];
 #pragma unroll
         for (int k = 0; k < DIM; ++k) first[k] = prev[k] = 0.f;
-        if (jb < je) {
-            float t1[1];
-            tp.get<1, true>(tm, jb, 1, je, t1);
-            e.eval(t1[0], first);
+        uint32_t jb, je;
+        if constexpr (PACKED) {
+            // two half runs a lane, in whole groups of 4 samples shared out evenly
+            const uint32_t ng = (n_t + 3) / 4, q = ng >> (lg + 1), r = ng & (2 * G - 1);
+            const uint32_t h0 = 2 * li, h1 = h0 + 1, h2 = h0 + 2;
+            jb = min(n_t, 4 * (h0 * q + min(h0, r)));
+            je = live ? min(n_t, 4 * (h2 * q + min(h2, r))) : jb;
+            const uint32_t jm = min(je, 4 * (h1 * q + min(h1, r)));
+            if (jb < je) acc = packed_run<D, DIM>(e, tp, jb, jm, je, first, prev);
+        } else {
+            jb = min(li * run, n_t);
+            je = live ? min(jb + run, n_t) : jb;
+            if (jb < je) {
+                float t1[1];
+                tp.get<1, true>(tm, jb, 1, je, t1);
+                e.eval(t1[0], first);
 #pragma unroll
-            for (int k = 0; k < DIM; ++k) prev[k] = first[k];
-        }
-        uint32_t j = jb + 1;
-        for (; j + 4 <= je; j += 4) {
-            // the group's 4 segments are summed first and then added to the run
-            float t[4], gs = 0.f;
-            tp.get<4, true>(tm, j, 1, je, t);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                float P[DIM];
-                e.eval(t[m], P);
-                gs += seg_len<DIM>(P, prev);
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) prev[k] = P[k];
+                for (int k = 0; k < DIM; ++k) prev[k] = first[k];
             }
-            acc += gs;
-        }
-        if (j < je) {
-            float t[4];
-            tp.get(tm, j, 1, je, t);
+            uint32_t j = jb + 1;
+            for (; j + 4 <= je; j += 4) {
+                // the group's 4 segments are summed first and then added to the run
+                float t[4], gs = 0.f;
+                tp.get<4, true>(tm, j, 1, je, t);
 #pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                if (j + m < je) {
+                for (int m = 0; m < 4; ++m) {
                     float P[DIM];
                     e.eval(t[m], P);
-                    acc += seg_len<DIM>(P, prev);
+                    gs += seg_len<DIM>(P, prev);
 #pragma unroll
                     for (int k = 0; k < DIM; ++k) prev[k] = P[k];
+                }
+                acc += gs;
+            }
+            if (j < je) {
+                float t[4];
+                tp.get(tm, j, 1, je, t);
+#pragma unroll
+                for (int m = 0; m < 3; ++m) {
+                    if (j + m < je) {
+                        float P[DIM];
+                        e.eval(t[m], P);
+                        acc += seg_len<DIM>(P, prev);
+#pragma unroll
+                        for (int k = 0; k < DIM; ++k) prev[k] = P[k];
+                    }
                 }
             }
         }
@@ -365,12 +546,17 @@ LaunchResult launch_points(const CurveArgs& a, int tm, cudaStream_t s, const Lau
 template <int VAR, int D, int DIM>
 LaunchResult launch_length(const CurveArgs& a, int tm, cudaStream_t s, const LaunchHooks& h)
 {
-    auto kern = k_length<VAR, D, DIM>;
+    constexpr bool PACKED = VAR == VAR_HORNER_CENTRED;  // the packed form serves the pre-mixed draw
+    const bool packed = PACKED && tm == TM_HASH16;
+    auto kern = packed ? k_length<VAR, D, DIM, PACKED> : k_length<VAR, D, DIM, false>;
     // runs of 16 to 32 samples a lane until a curve has a warp.  By n_t alone:
     // the order of the sum, and so a curve's length to the last bit, does not
     // depend on the other curves of the call.
+    // In-kernel draws of 64 samples and more take 4 lanes a curve: nothing is
+    // read per sample, and a lane's set-up and joins serve the longest runs.
     int lg = 2;
-    while (lg < 5 && a.n_t > (32 << lg)) ++lg;
+    if (!packed)
+        while (lg < 5 && a.n_t > (32 << lg)) ++lg;
     const int64_t units = (a.n_curves + (32 >> lg) - 1) / (32 >> lg);
     const int grid = tile_grid((const void*)kern, units, h.sm_count);
     h.count(h.self);
@@ -397,22 +583,15 @@ LaunchResult launch_dynamic(const CurveArgs& a, int tm, int om, cudaStream_t s, 
     return launch_one<VAR, 0, DIM, TM_HASH, OM_LENGTH>(a, s, h);
 }
 
-// Fixed degrees.  The fused draw-and-measure form of 3D curves has kernels of
-// its own (the pre-mixed draw needs every sample index below 2^16); the rest
-// runs k_points and k_length.
+// Fixed degrees: k_points and k_length (the pre-mixed draw needs every sample
+// index below 2^16).
 template <int VAR, int D, int DIM>
 LaunchResult launch_fixed(const CurveArgs& a, int tm, int om, cudaStream_t s, const LaunchHooks& h)
 {
     if (om == OM_POINTS) return launch_points<VAR, D, DIM>(a, tm, s, h);
     const bool draw16 = tm == TM_HASH && a.n_t <= 65536;
-    if constexpr (DIM == 3) {
-        // centred Horner up to degree 4 runs two curves per warp from 64
-        // samples, four from 128 and eight from 256
-        if constexpr (VAR == VAR_HORNER_CENTRED && D <= 4) {
-            if (draw16 && a.n_t >= kGroup4MinSamples) return launch_group<D, 4>(a, s, h);
-            if (draw16 && a.n_t >= kGroup8MinSamples) return launch_group<D, 8>(a, s, h);
-            if (draw16 && a.n_t >= 64) return launch_pair<D>(a, s, h);
-        }
+    // (the other evaluators' fused draw-and-measure form keeps a warp per curve)
+    if constexpr (DIM == 3 && VAR != VAR_HORNER_CENTRED) {
         if (draw16) return launch_one<VAR, D, DIM, TM_HASH16, OM_LENGTH>(a, s, h);
     }
     return launch_length<VAR, D, DIM>(a, draw16 ? TM_HASH16 : tm, s, h);
