@@ -3,10 +3,10 @@
 // between u, v and w; the bicubic case evaluates the four column curves at u
 // and then the isoline cubic in v).
 //
-// Separable contraction, one block per patch (grid-stride; bicubic 3D
-// patches on grids of up to 64 rows take one warp per patch, and tricubic
-// scalar volumes one warp per volume: k_volume_tricubic1_warp in
-// tensor_common.cuh, shared with the texture volumes):
+// Separable contraction (bicubic 3D patches on grids of up to 64 rows take one
+// warp per patch, larger ones a block; tricubic scalar volumes one warp per
+// volume: k_volume_tricubic1_warp in tensor_common.cuh, shared with the texture
+// volumes; every other grid k_grid, one warp per block of rows):
 //   surface  X[a][j] = sum_i Bu[a][i] C[i][j]          (isoline control points)
 //            P[a][b] = sum_j X[a][j] Bv[b][j]
 //   volume   Y[a][j][l] = sum_i Bu[a][i] C[i][j][l]
@@ -18,6 +18,7 @@
 // coalesced.  The contraction has a reduction depth of 4 for bicubic
 // patches, far too small to keep tensor cores busy on a store-bound kernel,
 // so it runs on the FP32 pipes.
+#include "curve_tile.cuh"
 #include "tensor_common.cuh"
 
 namespace bez {
@@ -170,126 +171,170 @@ __global__ void __launch_bounds__(kSurfWarps * 32, 5) k_surface_bicubic3_warp(co
     }
 }
 
-// General surfaces: any degrees <= 7, dim 1..4, grid <= 256 per axis.  One
-// thread per output point (strided), outputs staged in shared memory and
-// written as consecutive floats.
-__global__ void __launch_bounds__(kTensorThreads) k_surface_generic(const TensorArgs a)
+// General grids: any degrees <= 7, dim 1..4, grid <= 256 per axis.  One warp per
+// unit of work, a block of up to kGridRows rows of one u slab of one volume; a
+// surface is a volume of one slab (degree 0, one grid value) whose v and w are
+// its u and v.  The warp forms Y[j][k][l] = sum_i Bu[i] C[i][j][l][k] and
+// Z[b][k][l] = sum_j Bv[b][j] Y[j][k][l] in warp-private shared memory, l padded
+// to whole float4s, then takes the rows' points in output order, 4 a lane: a
+// point is L4 float4 products of Bw[c] and Z[b] a component, staged and written
+// as float4s.  (The block-per-volume kernel before it wrote each row from one
+// thread, 16 bytes every row length, with runtime inner loops.)  Bound by
+// instruction issue (64 %) and shared memory.  A call (us, GB300): 1000 tricubic
+// 3D lattices on 20 x 24 x 28 162 -> 46; 8000 on 5 x 30 x 7 147 -> 50; 30,000
+// bicubic patches on 32 x 33 356 -> 95, of degree 2 x 1 261 -> 79, 5 x 5
+// 364 -> 155.  4 blocks per SM (3 in 4D) measured best of 3 to 5.
+constexpr int kGridRows = 32;
+constexpr int kGridTile = 128;  // points a warp stages between two write-outs
+
+// shared memory in floats: the tables, then each warp's C, Y, Z and stage
+struct GridLayout {
+    int bv, bu, warp, c, y, z, per_warp, total;
+};
+__host__ __device__ inline GridLayout grid_layout(const TensorArgs& a)
 {
-    extern __shared__ float sm[];
-    const int du = a.du, dv = a.dv, dim = a.dim, nu = a.nu, nv = a.nv;
-    float* s_bu = sm;                                   // nu * (du+1)
-    float* s_bv = s_bu + nu * (du + 1);                 // nv * (dv+1)
-    float* s_c = s_bv + nv * (dv + 1);                  // (du+1)(dv+1)dim
-    float* s_x = s_c + (du + 1) * (dv + 1) * dim;       // nu * (dv+1) * dim
-    float* s_o = s_x + nu * (dv + 1) * dim;             // kTensorThreads * dim
-    const int tid = threadIdx.x;
-    bernstein_table(s_bu, nu, du, tid, kTensorThreads);
-    bernstein_table(s_bv, nv, dv, tid, kTensorThreads);
-    const int per = (du + 1) * (dv + 1) * dim;
-    const int64_t pts = (int64_t)nu * nv;
-    for (int64_t p = blockIdx.x; p < a.n; p += gridDim.x) {
-        __syncthreads();
-        for (int e = tid; e < per; e += kTensorThreads) s_c[e] = load_elem(a.ctrl, a.dtype, p * per + e);
-        __syncthreads();
-        const int xr = (dv + 1) * dim;
-        for (int e = tid; e < nu * xr; e += kTensorThreads) {
-            const int row = e / xr, jk = e - row * xr;
-            float x = 0.f;
-            for (int i = 0; i <= du; ++i) x = fmaf(s_bu[row * (du + 1) + i], s_c[i * xr + jk], x);
-            s_x[e] = x;
-        }
-        __syncthreads();
-        float* out = a.out + p * pts * dim;
-        for (int64_t q0 = 0; q0 < pts; q0 += kTensorThreads) {
-            const int64_t q = q0 + tid;
-            if (q < pts) {
-                const int row = (int)(q / nv), b = (int)(q - (int64_t)row * nv);
-                for (int k = 0; k < dim; ++k) {
-                    float v = 0.f;
-                    for (int j = 0; j <= dv; ++j) v = fmaf(s_bv[b * (dv + 1) + j], s_x[row * xr + j * dim + k], v);
-                    s_o[tid * dim + k] = v;
-                }
-            }
-            __syncthreads();
-            const int64_t valid = min((int64_t)kTensorThreads, pts - q0) * dim;
-            for (int f = tid; f < valid; f += kTensorThreads) out[q0 * dim + f] = s_o[f];
-            __syncthreads();
-        }
-    }
+    const int lw = a.dw > 3 ? 8 : 4;
+    GridLayout g;
+    g.bv = a.nw * lw;
+    g.bu = g.bv + a.nv * (a.dv + 1);
+    g.warp = (g.bu + a.nu * (a.du + 1) + 3) & ~3;
+    g.y = kGridTile * a.dim;  // after the stage
+    g.z = g.y + (a.dv + 1) * a.dim * lw;
+    g.c = g.z + kGridRows * a.dim * lw;
+    g.per_warp = (g.c + (a.du + 1) * (a.dv + 1) * (a.dw + 1) * a.dim + 3) & ~3;
+    g.total = g.warp + kSurfWarps * g.per_warp;
+    return g;
 }
 
-// Volumes (any degrees <= 7, dim 1..4): Y and Z stages in shared memory, one
-// thread per (a, b) line writing its nw * dim consecutive values.
-__global__ void __launch_bounds__(kTensorThreads) k_volume(const TensorArgs a)
+template <int L4, int DIM>
+__global__ void __launch_bounds__(kSurfWarps * 32, DIM == 4 ? 3 : 4) k_grid(const TensorArgs a, int chunks)
 {
-    extern __shared__ float sm[];
-    const int du = a.du, dv = a.dv, dw = a.dw, dim = a.dim, nu = a.nu, nv = a.nv, nw = a.nw;
-    float* s_bu = sm;
-    float* s_bv = s_bu + nu * (du + 1);
-    float* s_bw = s_bv + nv * (dv + 1);
-    float* s_c = s_bw + nw * (dw + 1);
-    const int per = (du + 1) * (dv + 1) * (dw + 1) * dim;
-    float* s_y = s_c + per;                                 // nu (dv+1) (dw+1) dim
-    float* s_z = s_y + nu * (dv + 1) * (dw + 1) * dim;      // nu nv (dw+1) dim
-    const int tid = threadIdx.x;
-    bernstein_table(s_bu, nu, du, tid, kTensorThreads);
-    bernstein_table(s_bv, nv, dv, tid, kTensorThreads);
-    bernstein_table(s_bw, nw, dw, tid, kTensorThreads);
-    const int lk = (dw + 1) * dim;                          // (l, k) entries of one (i, j)
-    const int64_t pts = (int64_t)nu * nv * nw;
-    for (int64_t p = blockIdx.x; p < a.n; p += gridDim.x) {
-        __syncthreads();
-        for (int e = tid; e < per; e += kTensorThreads) s_c[e] = load_elem(a.ctrl, a.dtype, p * per + e);
-        __syncthreads();
-        const int ny = nu * (dv + 1) * lk;
-        for (int e = tid; e < ny; e += kTensorThreads) {
-            const int row = e / ((dv + 1) * lk), jlk = e - row * ((dv + 1) * lk);
+    constexpr int LW = 4 * L4;
+    extern __shared__ float4 s_grid[];
+    float* sm = reinterpret_cast<float*>(s_grid);
+    const GridLayout g = grid_layout(a);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int du = a.du, dv = a.dv, dw = a.dw, nu = a.nu, nv = a.nv, nw = a.nw;
+    bernstein_table(sm, nw, dw, tid, kSurfWarps * 32, LW);
+    bernstein_table(sm + g.bv, nv, dv, tid, kSurfWarps * 32);
+    bernstein_table(sm + g.bu, nu, du, tid, kSurfWarps * 32);
+    __syncthreads();
+    const float4* bw4 = s_grid;
+    float* mine = sm + g.warp + (tid >> 5) * g.per_warp;
+    float *stage = mine, *Y = mine + g.y, *Z = mine + g.z, *C = mine + g.c;
+    const int ljk = (dw + 1) * DIM;  // floats of one (i, j)
+    const int per = (du + 1) * (dv + 1) * ljk;
+    const int q32 = 32 / nw, r32 = 32 - q32 * nw;  // 32 points on: q32 rows and r32 columns
+    // a warp takes consecutive units, most of them of one volume: its control
+    // points load once per volume, Y is formed once per slab
+    const int64_t n_units = a.n * nu * chunks, n_warps = (int64_t)gridDim.x * kSurfWarps;
+    const int64_t w = (int64_t)blockIdx.x * kSurfWarps + (tid >> 5), each = n_units / n_warps;
+    const int64_t more = n_units - each * n_warps;  // warps with one unit more
+    const int64_t u0 = w * each + min(w, more);
+    int64_t left = each + (w < more ? 1 : 0), slab = u0 / chunks, p = slab / nu, loaded = -1, formed = -1;
+    int ch = (int)(u0 - slab * chunks), ai = (int)(slab - p * nu);
+    for (; left > 0; --left) {
+        const int b0 = ch * kGridRows;
+        const int rows = min(kGridRows, nv - b0);
+        if (p != loaded) {
+            if (a.dtype == 0) {
+                const float* src = static_cast<const float*>(a.ctrl) + p * per;
+                for (int e = lane; e < per; e += 32) C[e] = __ldg(src + e);
+            } else {
+                for (int e = lane; e < per; e += 32) C[e] = load_elem(a.ctrl, a.dtype, p * per + e);
+            }
+            loaded = p;
+            __syncwarp();
+        }
+        const float* bu = sm + g.bu + ai * (du + 1);
+        for (int e = lane; e < (slab != formed ? (dv + 1) * DIM * LW : 0); e += 32) {
+            const int j = e / (DIM * LW), k = e / LW % DIM, l = e % LW;
             float y = 0.f;
-            for (int i = 0; i <= du; ++i) y = fmaf(s_bu[row * (du + 1) + i], s_c[i * (dv + 1) * lk + jlk], y);
-            s_y[e] = y;
+            if (l <= dw) {
+                const float* src = C + j * ljk + l * DIM + k;
+                for (int i = 0; i <= du; ++i) y = fmaf(bu[i], src[i * (dv + 1) * ljk], y);
+            }
+            Y[e] = y;
         }
-        __syncthreads();
-        const int nz = nu * nv * lk;
-        for (int e = tid; e < nz; e += kTensorThreads) {
-            const int ab = e / lk, l_k = e - ab * lk;
-            const int ai = ab / nv, b = ab - ai * nv;
-            float z = 0.f;
-            for (int j = 0; j <= dv; ++j)
-                z = fmaf(s_bv[b * (dv + 1) + j], s_y[(ai * (dv + 1) + j) * lk + l_k], z);
-            s_z[e] = z;
+        formed = slab;
+        __syncwarp();
+        for (int e = lane; e < rows * DIM * L4; e += 32) {
+            const int b = e / (DIM * L4), r = e - b * (DIM * L4);
+            const float* bv = sm + g.bv + (b0 + b) * (dv + 1);
+            const float4* y4 = reinterpret_cast<const float4*>(Y) + r;
+            float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int j = 0; j <= dv; ++j) {
+                const float4 y = y4[j * (DIM * L4)];
+                const float w = bv[j];
+                z.x = fmaf(w, y.x, z.x);
+                z.y = fmaf(w, y.y, z.y);
+                z.z = fmaf(w, y.z, z.z);
+                z.w = fmaf(w, y.w, z.w);
+            }
+            reinterpret_cast<float4*>(Z)[e] = z;
         }
-        __syncthreads();
-        float* out = a.out + p * pts * dim;
-        const int line = nw * dim;
-        if (line % 4 == 0 && (((uintptr_t)out) & 15) == 0) {
-            // one thread per (a, b) line: its nw * dim values as float4 stores
-            for (int ab = tid; ab < nu * nv; ab += kTensorThreads) {
-                float4* o = reinterpret_cast<float4*>(out + (int64_t)ab * line);
-                const float* z = s_z + ab * lk;
-                for (int f4 = 0; f4 < line / 4; ++f4) {
-                    float r[4];
-                    for (int m = 0; m < 4; ++m) {
-                        const int ck = f4 * 4 + m, c = ck / dim, k = ck - c * dim;
-                        float v = 0.f;
-                        for (int l = 0; l <= dw; ++l) v = fmaf(s_bw[c * (dw + 1) + l], z[l * dim + k], v);
-                        r[m] = v;
+        __syncwarp();
+        const int total = rows * nw;
+        float* out = a.out + ((slab * nv + b0) * (int64_t)nw) * DIM;
+        int b = lane / nw, c = lane - b * nw;
+        for (int t0 = 0; t0 < total; t0 += kGridTile) {
+            const int cnt = min(kGridTile, total - t0);
+#pragma unroll
+            for (int m = 0; m < kGridTile / 32; ++m) {
+                if (lane + 32 * m < cnt) {
+                    const float4* z4 = reinterpret_cast<const float4*>(Z) + b * (DIM * L4);
+                    float v[DIM];
+#pragma unroll
+                    for (int k = 0; k < DIM; ++k) v[k] = 0.f;
+#pragma unroll
+                    for (int q = 0; q < L4; ++q) {
+                        const float4 w = bw4[c * L4 + q];
+#pragma unroll
+                        for (int k = 0; k < DIM; ++k) {
+                            const float4 z = z4[k * L4 + q];
+                            v[k] = fmaf(w.x, z.x, v[k]);
+                            v[k] = fmaf(w.y, z.y, v[k]);
+                            v[k] = fmaf(w.z, z.z, v[k]);
+                            v[k] = fmaf(w.w, z.w, v[k]);
+                        }
                     }
-                    o[f4] = make_float4(r[0], r[1], r[2], r[3]);
+#pragma unroll
+                    for (int k = 0; k < DIM; ++k) stage[(lane + 32 * m) * DIM + k] = v[k];
+                }
+                b += q32;
+                c += r32;
+                if (c >= nw) {
+                    c -= nw;
+                    ++b;
                 }
             }
-        } else {
-            for (int e = tid; e < nu * nv * line; e += kTensorThreads) {
-                // consecutive threads write consecutive floats of the volume
-                const int ab = e / line, ck = e - ab * line;
-                const int c = ck / dim, k = ck - c * dim;
-                float v = 0.f;
-                for (int l = 0; l <= dw; ++l) v = fmaf(s_bw[c * (dw + 1) + l], s_z[ab * lk + l * dim + k], v);
-                out[e] = v;
+            __syncwarp();
+            tile_copy(out + (int64_t)t0 * DIM, stage, cnt * DIM, lane, 32);
+            __syncwarp();
+        }
+        if (++ch == chunks) {
+            ch = 0;
+            ++slab;
+            if (++ai == nu) {
+                ai = 0;
+                ++p;
             }
         }
     }
 }
 
+static const void* grid_kernel(int l4, int dim)
+{
+    switch (dim) {
+    case 1: return l4 == 1 ? (const void*)k_grid<1, 1> : (const void*)k_grid<2, 1>;
+    case 2: return l4 == 1 ? (const void*)k_grid<1, 2> : (const void*)k_grid<2, 2>;
+    case 3: return l4 == 1 ? (const void*)k_grid<1, 3> : (const void*)k_grid<2, 3>;
+    default: return l4 == 1 ? (const void*)k_grid<1, 4> : (const void*)k_grid<2, 4>;
+    }
+}
+
+// The shared memory of a block-per-patch form of the contraction, which bounds
+// the grids that are accepted (200 KB).
 size_t tensor_smem_bytes(const TensorArgs& a)
 {
     if (a.dw < 0) {
@@ -330,10 +375,12 @@ LaunchResult launch_tensor_product(const TensorLaunch& t, cudaStream_t s, const 
     size_t smem = 0;
     int threads = kTensorThreads;
     int64_t work = a.n;
+    int chunks = 1;
     const bool bicubic3 = a.dw < 0 && a.du == 3 && a.dv == 3 && a.dim == 3 && a.nv % 4 == 0 &&
                           ((uintptr_t)a.out & 15) == 0;
     const bool tricubic1 = a.dw == 3 && a.du == 3 && a.dv == 3 && a.dim == 1 && a.nu <= kVolMaxRows &&
                            a.nw % 4 == 0 && ((uintptr_t)a.out & 15) == 0;
+    const bool general = !bicubic3 && !tricubic1;
     if (bicubic3 && a.nu <= kSurfMaxRows) {
         kern = (const void*)k_surface_bicubic3_warp;
         threads = kSurfWarps * 32;
@@ -346,16 +393,29 @@ LaunchResult launch_tensor_product(const TensorLaunch& t, cudaStream_t s, const 
     } else if (bicubic3) {
         kern = (const void*)k_surface_bicubic3;
     } else {
-        kern = a.dw < 0 ? (const void*)k_surface_generic : (const void*)k_volume;
-        smem = tensor_smem_bytes(a);
+        if (a.dw < 0) {  // a surface: one slab, u and v in the places of v and w
+            a.dw = a.dv;
+            a.nw = a.nv;
+            a.dv = a.du;
+            a.nv = a.nu;
+            a.du = 0;
+            a.nu = 1;
+        }
+        kern = grid_kernel(a.dw > 3 ? 2 : 1, a.dim);
+        threads = kSurfWarps * 32;
+        chunks = (a.nv + kGridRows - 1) / kGridRows;
+        work = (a.n * a.nu * chunks + kSurfWarps - 1) / kSurfWarps;
+        smem = (size_t)grid_layout(a).total * sizeof(float);
         if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            // the most a launch of this kernel takes, so that calls on several
+            // threads never lower one another's limit
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
             if (e != cudaSuccess) return {0, e};
         }
     }
     const int grid = persistent_grid(kern, threads, smem, h.sm_count, work);
     const SurfTexArgs no_tex{};  // the CUDA-core volume kernel reads no texture
-    void* args[] = {(void*)&a, (void*)&no_tex};
+    void* args[] = {(void*)&a, general ? (void*)&chunks : (void*)&no_tex};
     h.count(h.self);
     h.begin(h.self, s);
     cudaError_t e = cudaLaunchKernel(kern, dim3(grid), dim3(threads), args, smem, s);

@@ -35,8 +35,10 @@ inline int volume_parts(int64_t n, int nu, int sm_count)
 
 // Bernstein table B[a][i] for n grid values and degree d, via de Casteljau
 // on unit vectors (each entry is a product of lerp weights, exact at ends).
-__device__ __forceinline__ void bernstein_table(float* B, int n, int d, int tid, int nthreads)
+// Rows of `stride` floats (d + 1 where 0), zeros after the d + 1 values.
+__device__ __forceinline__ void bernstein_table(float* B, int n, int d, int tid, int nthreads, int stride = 0)
 {
+    if (stride == 0) stride = d + 1;
     for (int a = tid; a < n; a += nthreads) {
         const float t = n > 1 ? __fdiv_rn((float)a, (float)(n - 1)) : 0.f;
         const float s = 1.0f - t;
@@ -49,9 +51,10 @@ __device__ __forceinline__ void bernstein_table(float* B, int n, int d, int tid,
         }
         float bin = 1.f;
         for (int i = 0; i <= d; ++i) {
-            B[a * (d + 1) + i] = bin * sp[d - i] * tp[i];
+            B[a * stride + i] = bin * sp[d - i] * tp[i];
             bin = bin * (float)(d - i) / (float)(i + 1);
         }
+        for (int i = d + 1; i < stride; ++i) B[a * stride + i] = 0.f;
     }
 }
 
