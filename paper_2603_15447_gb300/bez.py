@@ -92,6 +92,8 @@ _VP, _I64, _INT = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int
 def lib():
     """Load libbez.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lib_lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -139,9 +141,15 @@ def _check(st):
 
 # ---------------------------------------------------------------- marshalling
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _ptr(x):
@@ -160,9 +168,13 @@ def _is_cuda(x):
 
 
 def _stream_handle(stream, device):
-    torch = _torch()
     if stream is None:
-        return torch.cuda.current_stream(device).cuda_stream
+        torch = _torch()
+        if type(device) is not int:
+            return torch.cuda.current_stream(device).cuda_stream
+        # the handle alone: current_stream() builds a Stream object around it
+        # (3.5 us of an 18 us call)
+        return torch._C._cuda_getCurrentRawStream(device)
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -173,6 +185,8 @@ def _dtype_code(x):
         m = {np.dtype(np.float32): DType.F32, np.dtype(np.float16): DType.F16}
         return m[x.dtype]
     torch = _torch()
+    if x.dtype is torch.float32:
+        return DType.F32
     m = {torch.float32: DType.F32, torch.float16: DType.F16, torch.bfloat16: DType.BF16}
     if x.dtype not in m:
         raise TypeError(f"control points must be float32/float16/bfloat16, got {x.dtype}")
@@ -180,9 +194,11 @@ def _dtype_code(x):
 
 
 def _empty_like_location(ref, shape):
-    torch = _torch()
     if isinstance(ref, np.ndarray):
         return np.empty(shape, np.float32)
+    torch = _torch()
+    if type(ref) is torch.Tensor and ref.dtype is torch.float32:
+        return ref.new_empty(shape)  # (cheaper than naming dtype and device)
     return torch.empty(shape, dtype=torch.float32, device=ref.device)
 
 

@@ -1,6 +1,7 @@
 // api.cu -- host runtime of libbez.so: contexts, argument validation, host
 // staging, launch accounting and dispatch to the kernels.  The C ABI is
 // declared in include/bez.h.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cstdarg>
@@ -86,9 +87,37 @@ void hook_end(void* self, cudaStream_t s)
 
 LaunchHooks bez::hooks_of(bez_ctx c) { return LaunchHooks{hook_count, hook_begin, hook_end, c, c->sm_count}; }
 
+namespace {
+
+// cuPointerGetAttribute, or NULL: one attribute costs a fraction of the set
+// that cudaPointerGetAttributes collects, and every array of every call is asked
+CUresult (*pointer_attribute())(void*, CUpointer_attribute, CUdeviceptr)
+{
+    using Fn = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+    static const Fn fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Fn>(f);
+    }();
+    return fn;
+}
+
+}  // namespace
+
 bez::MemKind bez::classify(const void* p)
 {
     if (!p) return MEM_NULL;
+    if (auto fn = pointer_attribute()) {
+        unsigned type = 0;
+        if (fn(&type, CU_POINTER_ATTRIBUTE_MEMORY_TYPE, reinterpret_cast<CUdeviceptr>(p)) == CUDA_SUCCESS &&
+            type == CU_MEMORYTYPE_DEVICE)
+            return MEM_DEVICE;  // anything else is looked at in full
+    }
     cudaPointerAttributes at;
     cudaError_t e = cudaPointerGetAttributes(&at, p);
     if (e != cudaSuccess) {
@@ -387,8 +416,8 @@ bez_status bez_eval(bez_ctx c, const void* ctrl, int64_t n_curves, int degree, i
     // Host control points and host output on a register evaluator: run the
     // call as chunks whose copies in and out overlap the evaluation of the
     // neighbouring chunks (per-curve host parameters disable it).
-    const bool pipe = !tex && classify(ctrl) == MEM_HOST && classify(out) == MEM_HOST &&
-                      n_curves >= 2 * kPipeMinCurves && !(o->t_mode == BEZ_T_PER_CURVE && classify(t) == MEM_HOST);
+    const bool pipe = !tex && n_curves >= 2 * kPipeMinCurves && classify(ctrl) == MEM_HOST &&
+                      classify(out) == MEM_HOST && !(o->t_mode == BEZ_T_PER_CURVE && classify(t) == MEM_HOST);
     if (pipe) {
         st = ensure_stage(c, 0, ctrl_bytes, s);
         if (st != BEZ_OK) return st;
