@@ -21,7 +21,7 @@
 // current span in registers and reloading them only when the span changes;
 // results go through a padded per-warp shared-memory tile and out with
 // coalesced stores.  Degree and component count are compile-time in the
-// per-item dispatch for 3D curves.
+// per-item dispatch for 2D and 3D curves.
 #include "curve_eval.cuh"
 #include "spline.cuh"
 
@@ -223,13 +223,12 @@ __device__ __forceinline__ void span_eval(const float (&k)[P + 1][C], float tau,
     }
 }
 
-// one item of a 3D curve with compile-time degree P; C = 3 (integral) or 4
-// (rational, homogeneous)
-template <int P, int C, int REPR>
+// one item of a 2D or 3D curve with compile-time degree P (homogeneous points
+// when rational)
+template <int P, int DIM, bool RAT, int REPR>
 __device__ void item_fixed(const BatchArgs& a, const BatchItem& it, float* stage, int lane)
 {
-    constexpr bool RAT = C == 4;
-    constexpr int DIM = 3;
+    constexpr int C = RAT ? DIM + 1 : DIM;
     constexpr int LS = kRun * DIM + 1;  // padded per-lane stride of the tile
     const int n = it.n_samples;
     const bool spline = it.n_spans > 0;
@@ -294,9 +293,16 @@ __device__ void item_fixed(const BatchArgs& a, const BatchItem& it, float* stage
         // With lane = 24 r0 + o0 and a = o0 div 8, run = r0 + m + w and
         // offset = o0 + 8 m - 24 w where w = (a + m) div 3, so its staged
         // position is base + m (LS + 8) + w (LS - 24).
-        static_assert(kRun * DIM == 24 && LS == 25, "write-out index formula");
+        // In 2D a run is 16 floats: run 2 m + lane div 16, offset lane mod 16.
+        static_assert(kRun == 8 && (DIM == 2 || DIM == 3), "write-out index formula");
         const int valid = vs * DIM;
-        if (lr == 3) {
+        if (lr == 3 && DIM == 2) {
+            float* o = out + (int64_t)tb * DIM + lane;
+            const int base = (lane >> 4) * LS + (lane & 15);
+#pragma unroll
+            for (int m = 0; m < kRun * DIM; ++m)
+                if (32 * m + lane < valid) o[32 * m] = stage[base + 2 * m * LS];
+        } else if (lr == 3) {
             float* o = out + (int64_t)tb * DIM + lane;
             const int a3 = (lane % 24) / 8;
             const int base = (lane / 24) * LS + lane % 24;
@@ -306,11 +312,11 @@ __device__ void item_fixed(const BatchArgs& a, const BatchItem& it, float* stage
                 if (32 * m + lane < valid) o[32 * m] = stage[base + m * (LS + 8) + w * (LS - 24)];
             }
         } else {
-            // short runs: float f is component f mod 3 of sample f div 3,
+            // short runs: float f is component f mod DIM of sample f div DIM,
             // element (sample mod run) of lane (sample div run)'s run
             float* o = out + (int64_t)tb * DIM;
             for (int f = lane; f < valid; f += 32) {
-                const int smp = f / 3, q = f - 3 * smp;
+                const int smp = f / DIM, q = f - DIM * smp;
                 o[f] = stage[(smp >> lr) * LS + (smp & ((1 << lr) - 1)) * DIM + q];
             }
         }
@@ -377,11 +383,11 @@ __device__ void item_generic(const BatchArgs& a, const BatchItem& it, float* sta
     }
 }
 
-// Item classes: 3D curves get one kernel per (degree, integral / rational),
-// everything else the generic kernel; the host sorts items by class.
+// Item classes: 2D and 3D curves get one kernel per (degree, integral /
+// rational), everything else the generic kernel; the host sorts items by class.
 int batch_item_class(const bez_curve_desc& d, int dim)
 {
-    if (dim != 3) return kBatchClasses - 1;
+    if (dim != 2 && dim != 3) return kBatchClasses - 1;
     return (d.type == BEZ_CURVE_NURBS ? 7 : 0) + (d.degree - 1);
 }
 
@@ -407,7 +413,7 @@ __device__ __forceinline__ BatchItem load_item(const BatchArgs& a, int64_t i)
 // table.  Static schedule: warp w takes items w, w + n_warps, ... and reads
 // the record of its next item while it evaluates the current one; atomic
 // schedule: `grab` items at a time from this class's counter.
-template <int P, int C, int REPR>
+template <int P, int DIM, bool RAT, int REPR>
 __global__ void __launch_bounds__(256) k_batch_class(const BatchArgs a, int64_t first, int64_t count,
                                                      unsigned long long* counter)
 {
@@ -417,8 +423,8 @@ __global__ void __launch_bounds__(256) k_batch_class(const BatchArgs a, int64_t 
     float* stage = s_stage + wib * (32 * (kRun * a.dim + 1));
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     auto run = [&](const BatchItem& it) {
-        if (P == 0) item_generic<REPR>(a, it, stage, lane);
-        else item_fixed<(P > 0 ? P : 1), (C > 0 ? C : 3), REPR>(a, it, stage, lane);
+        if constexpr (P == 0) item_generic<REPR>(a, it, stage, lane);
+        else item_fixed<P, DIM, RAT, REPR>(a, it, stage, lane);
     };
     if (a.schedule == 0) {
         int64_t item = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
@@ -441,26 +447,32 @@ __global__ void __launch_bounds__(256) k_batch_class(const BatchArgs a, int64_t 
     }
 }
 
-template <int REPR>
-static const void* class_kernel(int cls)
+template <int DIM, bool RAT, int REPR>
+static const void* class_degree(int p)
 {
-    switch (cls) {
-    case 0: return (const void*)k_batch_class<1, 3, REPR>;
-    case 1: return (const void*)k_batch_class<2, 3, REPR>;
-    case 2: return (const void*)k_batch_class<3, 3, REPR>;
-    case 3: return (const void*)k_batch_class<4, 3, REPR>;
-    case 4: return (const void*)k_batch_class<5, 3, REPR>;
-    case 5: return (const void*)k_batch_class<6, 3, REPR>;
-    case 6: return (const void*)k_batch_class<7, 3, REPR>;
-    case 7: return (const void*)k_batch_class<1, 4, REPR>;
-    case 8: return (const void*)k_batch_class<2, 4, REPR>;
-    case 9: return (const void*)k_batch_class<3, 4, REPR>;
-    case 10: return (const void*)k_batch_class<4, 4, REPR>;
-    case 11: return (const void*)k_batch_class<5, 4, REPR>;
-    case 12: return (const void*)k_batch_class<6, 4, REPR>;
-    case 13: return (const void*)k_batch_class<7, 4, REPR>;
-    default: return (const void*)k_batch_class<0, 0, REPR>;
+    switch (p) {
+    case 1: return (const void*)k_batch_class<1, DIM, RAT, REPR>;
+    case 2: return (const void*)k_batch_class<2, DIM, RAT, REPR>;
+    case 3: return (const void*)k_batch_class<3, DIM, RAT, REPR>;
+    case 4: return (const void*)k_batch_class<4, DIM, RAT, REPR>;
+    case 5: return (const void*)k_batch_class<5, DIM, RAT, REPR>;
+    case 6: return (const void*)k_batch_class<6, DIM, RAT, REPR>;
+    default: return (const void*)k_batch_class<7, DIM, RAT, REPR>;
     }
+}
+
+template <int REPR>
+static const void* class_kernel_of(int cls, int dim)
+{
+    if (cls == kBatchClasses - 1) return (const void*)k_batch_class<0, 0, false, REPR>;
+    const int p = cls % 7 + 1;
+    if (dim == 2) return cls < 7 ? class_degree<2, false, REPR>(p) : class_degree<2, true, REPR>(p);
+    return cls < 7 ? class_degree<3, false, REPR>(p) : class_degree<3, true, REPR>(p);
+}
+
+static const void* class_kernel(const BatchArgs& a, int cls)
+{
+    return a.repr == 1 ? class_kernel_of<1>(cls, a.dim) : class_kernel_of<0>(cls, a.dim);
 }
 
 static size_t batch_smem(const BatchArgs& a, int threads)
@@ -470,7 +482,7 @@ static size_t batch_smem(const BatchArgs& a, int threads)
 
 int batch_full_grid(const BatchArgs& a, int threads, int sm_count, int cls)
 {
-    const void* kern = a.repr == 1 ? class_kernel<1>(cls) : class_kernel<0>(cls);
+    const void* kern = class_kernel(a, cls);
     const int64_t count = a.class_start[cls + 1] - a.class_start[cls];
     const int wpb = threads / 32;
     return persistent_grid(kern, threads, batch_smem(a, threads), sm_count, (count + wpb - 1) / wpb);
@@ -534,7 +546,7 @@ cudaError_t launch_batch(const BatchArgs& a, int threads, int sm_count, bool wit
         cudaStream_t cs = lane_of == 0 ? s : bs->side[lane_of - 1];
         if (split_setup && (e = launch_setup(a, rec0, n_rec, sm_count, cs, h, launches)) != cudaSuccess) break;
         if (count <= 0) continue;
-        const void* kern = a.repr == 1 ? class_kernel<1>(cls) : class_kernel<0>(cls);
+        const void* kern = class_kernel(a, cls);
         const int wpb = threads / 32;
         int grid = persistent_grid(kern, threads, smem, sm_count, (count + wpb - 1) / wpb);
         if (part && a.class_grid[cls] > 0) grid = a.class_grid[cls];
