@@ -238,11 +238,14 @@ bez_status bez_eval_piecewise(bez_ctx ctx, const void* ctrl, int64_t n_chains, i
  *
  * Paper Sec. 2.2: B-splines become piecewise Bezier curves by Boehm's knot
  * insertion, and rational curves divide one integral spline point by
- * another (homogeneous coordinates).  A setup kernel extracts the Bezier
- * control points of every span in FP64 (one thread per span; rational
- * curves in homogeneous form (w P, w)) into a library-owned scratch buffer;
- * the evaluator finds each parameter's span, runs FP32 de Casteljau on it
- * and, for NURBS, divides by the weight.
+ * another (homogeneous coordinates).  The Bezier control points of every
+ * span are extracted (one thread per span; rational curves in homogeneous
+ * form (w P, w)) to more than FP32 precision and rounded once: in shared
+ * memory of the evaluating kernel up to degree 5 where a curve's spans fit
+ * it (float-float arithmetic), by a setup kernel in FP64 into a
+ * library-owned scratch buffer otherwise.  The evaluator finds each
+ * parameter's span, runs FP32 de Casteljau on it and, for NURBS, divides by
+ * the weight.
  *
  *   ctrl     [n_curves][n_ctrl][dim] FP32 (opts->dtype must be BEZ_F32)
  *   weights  [n_curves][n_ctrl] FP32 (NURBS only; positive weights expected)
@@ -273,8 +276,9 @@ bez_status bez_eval_nurbs(bez_ctx ctx, const float* ctrl, const float* weights, 
  * the isoline cubic in v); a volume splits it between u, v and w.  The
  * kernels contract separably (columns at u, then v, then w) with Bernstein
  * tables of the grid values fl32(a)/fl32(n-1) (one warp per patch for
- * bicubic 3D patches with nu <= 64, else one block per patch), and write
- * the output with coalesced (float4 where aligned) stores.
+ * bicubic 3D patches with nu <= 64 and nv a multiple of 4, one warp per
+ * block of grid rows otherwise), and write the output with coalesced
+ * (float4 where aligned) stores.
  *
  *   surface ctrl [n][du+1][dv+1][dim]        -> out [n][nu][nv][dim]
  *   volume  ctrl [n][du+1][dv+1][dw+1][dim]  -> out [n][nu][nv][nw][dim]
