@@ -6,7 +6,8 @@ namespace bez {
 
 bool spline_fits_fused(const SplineArgs& a)
 {
-    if (a.degree > kFusedMaxDegree || a.n_ctrl > 100000) return false;
+    // (a block per curve at worst: the curves have to fit a grid)
+    if (a.degree > kFusedMaxDegree || a.n_ctrl > 100000 || a.n_curves > 2147483647) return false;
     const FusedLayout f = fused_layout(1, a.n_ctrl, a.degree, a.dim, a.weights != nullptr, a.knots != nullptr);
     return (size_t)f.total * sizeof(float) <= kFusedMaxSmem;
 }
