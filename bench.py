@@ -59,15 +59,15 @@ T_OPS, LEN_OPS = 9, 8
 
 # DRAM bytes (read + write) per launch from one ncu capture of the current
 # kernels, per unit of work; null in the JSON line for other kernels.  The
-# curve kernel was captured on 131,072 curves (6,307,584 B: the control
+# curve kernel was captured on 131,072 curves (6,330,624 B: the control
 # points; the 4 B lengths stay in L2) and scales with the curve count; the
 # surface kernel on the full 65,536-patch tensor workload; the fused adjoint
 # on the full 65,536 x 512 fit step.
-TRAFFIC_PER_CURVE = {"HORNER_CENTRED": 6312448 / 131072}
+TRAFFIC_PER_CURVE = {"HORNER_CENTRED": 6330624 / 131072}
 # the kernel behind each headline variant's fused length (cubic 3D, hashed t)
 KERNEL_NAME = {"HORNER_CENTRED": "k_length<2, 3, 3, true> (four lanes per curve, two samples per instruction)", "HALF2": "k_curve_h2"}
 TRAFFIC_SURFACE_65536 = 12652544 + 742988544
-TRAFFIC_FIT_65536x512 = 540180736 + 121996800
+TRAFFIC_FIT_65536x512 = 540096000 + 120747776
 EVAL_OPS = {"HORNER": 9, "HORNER_CENTRED": 9, "HALF2": 5, "BERNSTEIN": 19, "SEILER": 16, "DECASTELJAU": 36,
             "TEX_DECASTELJAU": 3, "TEX_SEILER": 3, "TEX_HYBRID": 10, "TEX_SEILER_S8": 3, "TEX_SEILER_S4": 3}
 # filtered fetches per point and the peak they are held to
