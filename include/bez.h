@@ -340,8 +340,12 @@ bez_status bez_eval_volume(bez_ctx ctx, const void* ctrl, int64_t n, int du, int
  * file), and captures span setup + evaluation in a CUDA graph.
  * bez_batch_launch replays it on `stream`; with setup_each_launch = 0 the
  * spans are extracted once at creation (control points must then not
- * change).  bez_eval_batch is create + launch + destroy without graph or
- * tuning, synchronous on `stream`.
+ * change).  A plan with an atomic work queue and without a graph keeps one
+ * set of queue counters: order its launches (one stream, or an event between
+ * them).  Launches of a graph follow one another by themselves, and launches
+ * with the static schedule, the default without a graph, may overlap.
+ * bez_eval_batch is create + launch + destroy without graph or tuning,
+ * synchronous on `stream`.
  */
 typedef enum bez_curve_type { BEZ_CURVE_BEZIER = 0, BEZ_CURVE_BSPLINE = 1, BEZ_CURVE_NURBS = 2 } bez_curve_type;
 

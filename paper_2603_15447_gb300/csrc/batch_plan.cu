@@ -638,15 +638,22 @@ bez_status bez_batch_create(bez_ctx c, const bez_curve_desc* desc, int64_t n_cur
     // samples: short chunks leave a small batch enough items for every warp, and
     // long ones from an atomic queue a large one less overhead per item and an
     // even end (us of a launch, GB300, against static 512 / 256: 262,144 curves,
-    // 1.9e8 samples 865 / 923; 20,000 curves, 1.5e7 102 / 105; 3000 curves, 1.3e6
-    // 42.5 / 47.6).
+    // 1.9e8 samples 865 / 923; 80,000, 5.9e7 295 / 304; 20,000, 1.5e7 102 / 105;
+    // 3000, 1.3e6 42.5 / 47.6).
+    // The queue's counters are one set per plan.  Launches of a plan's graph follow
+    // one another, but without a graph two launches on different streams may
+    // overlap, and would then share out one queue: the static schedule, where every
+    // launch evaluates all items itself, is the default there.
     Shape sh;
-    sh.threads = 128;
     if (total_samples >= 60000000) {
-        sh.chunk = 1024;
-        sh.schedule = 1;
-    } else if (total_samples < 4000000) {
-        sh.chunk = 256;
+        if (b->use_graph) {
+            sh.threads = 128;
+            sh.chunk = 1024;
+            sh.schedule = 1;
+        }
+    } else {
+        sh.threads = 128;
+        if (total_samples < 4000000) sh.chunk = 256;
     }
     if (bo && bo->chunk > 0) sh.chunk = bo->chunk;
     if (bo && (bo->schedule == 0 || bo->schedule == 1)) sh.schedule = bo->schedule;
