@@ -635,25 +635,28 @@ bez_status bez_batch_create(bez_ctx c, const bez_curve_desc* desc, int64_t n_cur
              log2_bucket(n_curves ? (double)total_samples / n_curves : 0.0));
     b->key = key;
     // launch shape: explicit, tuned or default.  The default goes by the batch's
-    // samples: short chunks leave a small batch enough items for every warp, and
-    // long ones from an atomic queue a large one less overhead per item and an
-    // even end (us of a launch, GB300, against static 512 / 256: 262,144 curves,
-    // 1.9e8 samples 865 / 923; 80,000, 5.9e7 295 / 304; 20,000, 1.5e7 102 / 105;
-    // 3000, 1.3e6 42.5 / 47.6).
+    // samples: short chunks leave a small batch enough items for every warp, long
+    // ones cost a large one less per item.  us of a launch, GB300, chunks of 512 /
+    // 1024 / 2048 from the static schedule and 1024 from the atomic queue, blocks of
+    // 128 (256 threads: 1 to 3 % slower throughout):
+    //   3D 1.5e7 samples 101 / 109 / 128 / 189, 4.4e7 228 / 225 / 235 / 289, 7.3e7
+    //   364 / 358 / 361 / 395, 1.1e8 527 / 517 / 514 / 535, 1.5e8 698 / 676 / 671 /
+    //   674, 1.9e8 897 / 875 / 868 / 861; 2D 7.3e7 299 / 295 / 300 / 336, 1.9e8 739 /
+    //   719 / 714 / 709; curves of up to 1000 samples, 6.2e7 555 / 552 / 554 / 579;
+    //   of up to 16,384, 7e7 249 / 242 / 248 / 299; 3000 curves, 1.3e6: 256 42.5,
+    //   512 47.6
     // The queue's counters are one set per plan.  Launches of a plan's graph follow
     // one another, but without a graph two launches on different streams may
     // overlap, and would then share out one queue: the static schedule, where every
     // launch evaluates all items itself, is the default there.
     Shape sh;
-    if (total_samples >= 60000000) {
-        if (b->use_graph) {
-            sh.threads = 128;
-            sh.chunk = 1024;
-            sh.schedule = 1;
-        }
-    } else {
-        sh.threads = 128;
-        if (total_samples < 4000000) sh.chunk = 256;
+    sh.threads = 128;
+    if (total_samples < 4000000) sh.chunk = 256;
+    else if (total_samples >= 100000000) sh.chunk = 2048;
+    else if (total_samples >= 40000000) sh.chunk = 1024;
+    if (total_samples >= 160000000 && b->use_graph) {
+        sh.chunk = 1024;
+        sh.schedule = 1;
     }
     if (bo && bo->chunk > 0) sh.chunk = bo->chunk;
     if (bo && (bo->schedule == 0 || bo->schedule == 1)) sh.schedule = bo->schedule;
