@@ -384,7 +384,8 @@ __device__ void item_generic(const BatchArgs& a, const BatchItem& it, float* sta
 }
 
 // Item classes: 2D and 3D curves get one kernel per (degree, integral /
-// rational), everything else the generic kernel; the host sorts items by class.
+// rational), everything else (and `dim` 0, a small 2D plan) the generic kernel;
+// the host sorts items by class.
 int batch_item_class(const bez_curve_desc& d, int dim)
 {
     if (dim != 2 && dim != 3) return kBatchClasses - 1;

@@ -108,6 +108,7 @@ struct bez_batch_s {
     BatchItem* d_items = nullptr;
     size_t items_cap = 0;
     std::vector<int64_t> hspan_off;   // per curve, floats into the span pool
+    int class_dim = 0;                // dimension that the items are classed by (0: one class for all)
     BatchStreams streams{};
     bool have_streams = false;
     float* d_spans = nullptr;
@@ -153,7 +154,7 @@ bez_status build_items(bez_batch b, int chunk, cudaStream_t s)
     for (size_t c = 0; c < b->hdesc.size(); ++c) {
         const bez_curve_desc& d = b->hdesc[c];
         const int n = d.n_samples;
-        auto& v = per_class[batch_item_class(d, b->a.dim)];
+        auto& v = per_class[batch_item_class(d, b->class_dim)];
         for (int k = 0; (int64_t)k * chunk < n; ++k) {
             BatchItem it{};
             it.j0 = k * chunk;
@@ -431,7 +432,7 @@ bez_status bez_batch_create(bez_ctx c, const bez_curve_desc* desc, int64_t n_cur
     std::vector<int64_t> span_ops;                       // per span: offset of its matrix in ops
     std::vector<double> ops;
     std::vector<std::pair<int64_t, int>> mats;           // (offset, degree) of every distinct matrix
-    int64_t spans = 0, total_samples = 0, n_type[3] = {0, 0, 0}, deg_sum = 0;
+    int64_t spans = 0, total_samples = 0, items256 = 0, n_type[3] = {0, 0, 0}, deg_sum = 0;
     for (int64_t i = 0; i < n_curves; ++i) {
         const bez_curve_desc& d = b->hdesc[(size_t)i];
         const char* why = nullptr;
@@ -451,6 +452,7 @@ bez_status bez_batch_create(bez_ctx c, const bez_curve_desc* desc, int64_t n_cur
         n_type[d.type] += 1;
         deg_sum += d.degree;
         total_samples += d.n_samples;
+        items256 += ((int64_t)d.n_samples + 255) / 256;
         const int comps = d.type == BEZ_CURVE_NURBS ? dim + 1 : dim;
         const int n_spans = d.type == BEZ_CURVE_BEZIER ? 1 : d.n_ctrl - d.degree;
         span_off[(size_t)i] = spans;
@@ -488,6 +490,12 @@ bez_status bez_batch_create(bez_ctx c, const bez_curve_desc* desc, int64_t n_cur
             op_off[(size_t)i] = it->second;
         }
     }
+    // A small 2D batch keeps the generic kernel: one launch beside the extraction
+    // instead of two per class.  Its items are 256 samples then, and up to about
+    // 4000 of them run at once.  us of a launch, GB300, against the classes: 1000
+    // curves of up to 64 samples 29.0 / 30.6, 256 28.8 / 35.5, 1500 28.9 / 35.3; 4000
+    // of up to 256 33.3 / 39.1; 5000 of up to 64 47.2 / 33.3; 30 of up to 64 28.6 / 26.9.
+    b->class_dim = dim == 2 && items256 >= 64 && items256 <= 4000 && !(bo && bo->chunk > 256) ? 0 : dim;
     // plan-owned device buffers
     cudaError_t e = cudaSuccess;
     auto alloc = [&](void** p, size_t bytes) {
@@ -545,7 +553,7 @@ bez_status bez_batch_create(bez_ctx c, const bez_curve_desc* desc, int64_t n_cur
     for (int64_t i = 0; i < n_curves; ++i) order[(size_t)i] = i;
     auto span_key = [&](int64_t i) {
         const bez_curve_desc& d = b->hdesc[(size_t)i];
-        return ((int64_t)batch_item_class(d, dim) * 64 + d.degree) * 4 + d.type;
+        return ((int64_t)batch_item_class(d, b->class_dim) * 64 + d.degree) * 4 + d.type;
     };
     std::stable_sort(order.begin(), order.end(),
                      [&](int64_t x, int64_t y) { return span_key(x) < span_key(y); });
@@ -555,7 +563,7 @@ bez_status bez_batch_create(bez_ctx c, const bez_curve_desc* desc, int64_t n_cur
         int cls_next = 0;
         for (int64_t i : order) {
             const bez_curve_desc& d = b->hdesc[(size_t)i];
-            const int cls = batch_item_class(d, dim);
+            const int cls = batch_item_class(d, b->class_dim);
             while (cls_next <= cls) span_class_start[cls_next++] = (int64_t)span_rec.size();
             {
                 const bool spline = d.type != BEZ_CURVE_BEZIER, rat = d.type == BEZ_CURVE_NURBS;
