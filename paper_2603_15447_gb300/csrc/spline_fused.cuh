@@ -87,6 +87,10 @@ __device__ __forceinline__ bool extract_span_f2(const float* ctrl, const float* 
     const int comps = w ? dim + 1 : dim;
     constexpr int STEPS = P > 1 ? P * (P + 1) / 2 - 1 : 1;  // of either pass
     F2 al[STEPS], be[STEPS];
+    // steps of weight 1 (b is already an argument: clamped ends, repeated knots),
+    // which keep their point as the FP64 form does.  a + 1 (b - a) would lose a
+    // point beside one 2^22 times its size.  (Weight 0 returns a as it is.)
+    unsigned kept = 0;
     {
         const float a = s[P], b = s[P + 1];
         int k = 0;
@@ -98,7 +102,10 @@ __device__ __forceinline__ bool extract_span_f2(const float* ctrl, const float* 
 #pragma unroll
         for (int l = 1; l <= P - 1; ++l)
 #pragma unroll
-            for (int i = P; i >= l; --i) be[k++] = knot_ratio(b, a, s[P + i - l + 1], a);
+            for (int i = P; i >= l; --i, ++k) {
+                be[k] = knot_ratio(b, a, s[P + i - l + 1], a);
+                kept |= s[P + i - l + 1] == b ? 1u << k : 0u;
+            }
     }
     bool fine = true;
 #pragma unroll 1
@@ -122,7 +129,10 @@ __device__ __forceinline__ bool extract_span_f2(const float* ctrl, const float* 
 #pragma unroll
         for (int l = 1; l <= P - 1; ++l)
 #pragma unroll
-            for (int i = P; i >= l; --i, ++k) Q[i] = lerp2(Q[i - 1], Q[i], be[k]);
+            for (int i = P; i >= l; --i, ++k) {
+                const F2 v = lerp2(Q[i - 1], Q[i], be[k]);
+                Q[i] = (kept >> k) & 1u ? Q[i] : v;
+            }
 #pragma unroll
         for (int i = 0; i <= P; ++i) {
             const float v = __fadd_rn(Q[i].h, Q[i].l);
