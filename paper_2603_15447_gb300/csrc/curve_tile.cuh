@@ -35,7 +35,8 @@ static __device__ const CentredRows kCentredRows = make_centred_rows();
 // by `stride`).  Plain FP32 up to degree 4; from degree 5 the compensated dot
 // product of Ogita, Rump & Oishi (Dot2, 2005: products split exactly by fma,
 // partial sums by Knuth's TwoSum), which is as accurate as summing in twice
-// the precision and rounding once, at FP32 rate (FP64 runs at 1/64 of it).
+// the precision and rounding once, at FP32 rate (FP64 runs at 1/64 of it).  A sum
+// comes out infinite or NaN where a term leaves the FP32 range.
 template <int D>
 __device__ __forceinline__ float centred_entry(const float* b, int stride, int m)
 {
@@ -58,8 +59,7 @@ __device__ __forceinline__ float centred_entry(const float* b, int stride, int m
             sh = s;
             corr = __fadd_rn(corr, __fadd_rn(err, e));
         }
-        const float r = __fadd_rn(sh, corr);
-        return isfinite(sh) ? r : sh;  // an infinite or NaN sum has no correction
+        return __fadd_rn(sh, corr);
     }
 }
 
@@ -91,9 +91,24 @@ __device__ __forceinline__ void tile_setup(const CurveArgs& a, TileSmem<D, DIM, 
     __syncwarp();
     const int g = grp < nc ? grp : nc - 1;  // lanes without a curve follow the last one
     if constexpr (VAR == VAR_HORNER_CENTRED) {
+        bool fine = true;
         for (int i = lane; i < nc * PER; i += 32) {
             const int cc = i / PER, r = i - cc * PER, m = r / DIM, k = r - m * DIM;
-            sm.coef[i] = centred_entry<D>(sm.stage + cc * PER + k, DIM, m);
+            const float v = centred_entry<D>(sm.stage + cc * PER + k, DIM, m);
+            if (D >= kFp64SetupCentred) fine = fine && isfinite(v);
+            sm.coef[i] = v;
+        }
+        if (D >= kFp64SetupCentred && __any_sync(kFull, !fine)) {
+            // terms are up to 35 times a point and cancel: such a coefficient again in FP64
+#pragma unroll 1
+            for (int i = lane; i < nc * PER; i += 32) {
+                const int cc = i / PER, r = i - cc * PER, m = r / DIM, k = r - m * DIM;
+                double acc = 0.0;
+#pragma unroll 1
+                for (int j = 0; j <= D; ++j)
+                    acc = fma((double)__ldg(&kCentredRows.t[D][m][j]), (double)sm.stage[cc * PER + j * DIM + k], acc);
+                if (!isfinite(sm.coef[i])) sm.coef[i] = (float)acc;
+            }
         }
         __syncwarp();
         e.d = D;
