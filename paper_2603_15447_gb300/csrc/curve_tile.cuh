@@ -1,7 +1,7 @@
 // curve_tile.cuh -- the general register kernels for single curves of fixed
-// degree (1..7) and any dimension: points (k_points) and polyline lengths
-// (k_length), several curves per warp, and the fused draw-and-measure form of
-// centred Horner in packed FP32 pairs.
+// degree (1..7) and any dimension: points (k_points; k_points_few for small
+// calls) and polyline lengths (k_length), several curves per warp, and the fused
+// draw-and-measure form of centred Horner in packed FP32 pairs.
 //
 // The parameter kind (array, uniform grid, draw) is a launch argument: a lane
 // fetches the parameters of four samples behind one uniform branch, so one
@@ -250,6 +250,76 @@ __global__ void __launch_bounds__(kWarps * 32, (D + 1) * DIM > 20 ? 3 : (D + 1) 
             else if (live) tile_copy(o + grp * (int64_t)n_t * DIM, seg, ns * DIM, li, G);
             __syncwarp();
         }
+    }
+}
+
+// The evaluator of one curve from its control points in registers, with
+// tile_setup's arithmetic (centred Horner: below degree 5).
+template <int VAR, int D, int DIM>
+__device__ __forceinline__ void register_setup(const float (&b)[D + 1][DIM], Eval<VAR, D, DIM>& e)
+{
+    if constexpr (VAR == VAR_HORNER_CENTRED) {
+        static_assert(D < kFp64SetupCentred, "plain FP32 sums");
+        constexpr CentredMatrix<D> T = make_centred_matrix<D>();
+        e.d = D;
+#pragma unroll
+        for (int m = 0; m <= D; ++m)
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) {
+                float acc = 0.f;
+#pragma unroll
+                for (int i = 0; i <= D; ++i) acc = fmaf(T.t[m][i], b[i][k], acc);
+                e.a[m][k] = acc;
+            }
+    } else {
+        e.setup(b, D);
+    }
+}
+
+constexpr int kFewThreads = 128;
+
+// Points of a small call, one thread per sample or few: the curve's points come
+// straight into registers, beside the parameter, and nothing is staged, so that
+// a call is one load latency long instead of three.  Thread (c, q) takes samples
+// q, q + per, q + 2 per, ... of curve c, `per` threads a curve.
+template <int VAR, int D, int DIM>
+__global__ void __launch_bounds__(kFewThreads) k_points_few(const CurveArgs a, int tm, uint32_t per, uint32_t total)
+{
+    const uint32_t i = blockIdx.x * kFewThreads + threadIdx.x;
+    if (i >= total) return;
+    const uint32_t n_t = (uint32_t)a.n_t, c = i / per;
+    uint32_t j = i - c * per;
+    float t = 0.f, b[D + 1][DIM], P[DIM];
+    const float* tc = a.t + c * a.t_stride;
+    if (tm == TM_ARRAY) t = __ldg(tc + j);
+    const int64_t at = (int64_t)c * ((D + 1) * DIM);
+    if (a.dtype == 0) {
+#pragma unroll
+        for (int m = 0; m <= D; ++m)
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) b[m][k] = __ldg(static_cast<const float*>(a.ctrl) + at + m * DIM + k);
+    } else {
+#pragma unroll
+        for (int m = 0; m <= D; ++m)
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) b[m][k] = load_elem(a.ctrl, a.dtype, at + m * DIM + k);
+    }
+    Eval<VAR, D, DIM> e;
+    register_setup<VAR, D, DIM>(b, e);
+    const uint32_t key = curve_key<TM_HASH>(a, c);
+    const float den = (float)(n_t - 1);
+    float* o = a.out + (int64_t)c * n_t * DIM;
+    for (;;) {
+        float x = clamp01(t);
+        const uint32_t next = j + per;
+        if (tm == TM_ARRAY) t = next < n_t ? __ldg(tc + next) : 0.f;
+        else if (tm == TM_UNIFORM) x = n_t > 1 ? __fdiv_rn((float)j, den) : 0.f;
+        else x = hash_unit(lowbias32(key ^ j));
+        e.eval(x, P);
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) o[j * DIM + k] = P[k];
+        if (next >= n_t) break;
+        j = next;
     }
 }
 
@@ -529,6 +599,33 @@ inline int tile_grid(const void* kern, int64_t units, int sm_count)
 template <int VAR, int D, int DIM>
 LaunchResult launch_points(const CurveArgs& a, int tm, cudaStream_t s, const LaunchHooks& h)
 {
+    // Small calls (centred Horner from degree 5 on shares its compensated set-up
+    // over a curve's lanes, and keeps k_points).  us on GB300, k_points against
+    // k_points_few with 1, 2 and 4 samples a thread, FP32, shared t: cubics 100 x 64
+    // 2.9: 1.4; 1953 x 64 3.3: 2.1, 2.2, 2.4; 7812 x 64 5.5: 4.2, 3.3, 3.1; 15,625 x
+    // 64 8.7: 6.6, 4.8, 4.3; 3906 x 256 5.2: 6.6, 4.8, 4.2; 62,500 x 64 12.8: 22.4,
+    // 14.9, 11.5; 15,625 x 256 11.7: 22.2, 14.7, 11.0, with 8 samples 9.5; 125,000 x 8
+    // 9.5: 6.7, 5.4, 9.8; 166,666 x 24 14.6: 22.7, 15.3, 18.3.  4D quartics 10,000 x
+    // 100 7.9: 8.5, 6.7; 40,000 x 100 17.1: 29.7, 20.5, 19.4; 4D Bernstein of degree 7
+    // 62,500 x 8 10.5: 9.4; 125,000 x 8 13.2: 16.9.
+    const int64_t samples = a.n_curves * (int64_t)a.n_t;
+    constexpr int64_t kMost = DIM == 4 ? 1000000 : 4000000, kMostShort = DIM == 4 ? 500000 : 1000000;
+    if constexpr (VAR != VAR_HORNER_CENTRED || D < kFp64SetupCentred) {
+        if (samples <= (a.n_t >= 64 ? kMost : kMostShort)) {
+            const bool long_curves = a.n_t >= 256;
+            const uint32_t run = samples <= 200000                           ? 1
+                                 : samples <= (long_curves ? 600000 : 1000000)  ? 2
+                                 : samples <= 2000000 || !long_curves           ? 4
+                                                                               : 8;
+            const uint32_t per = ((uint32_t)a.n_t + run - 1) / run, total = (uint32_t)a.n_curves * per;
+            h.count(h.self);
+            h.begin(h.self, s);
+            k_points_few<VAR, D, DIM><<<(total + kFewThreads - 1) / kFewThreads, kFewThreads, 0, s>>>(a, tm, per, total);
+            const cudaError_t err = cudaGetLastError();
+            h.end(h.self, s);
+            return {1, err};
+        }
+    }
     auto kern = k_points<VAR, D, DIM>;
     // As few lanes per curve as hold its samples in one tile (8 a lane), 16 at
     // most, so that a lane's setup serves 8 samples and more; more lanes when
