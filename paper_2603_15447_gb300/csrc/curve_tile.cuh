@@ -276,6 +276,24 @@ __device__ __forceinline__ void register_setup(const float (&b)[D + 1][DIM], Eva
     }
 }
 
+// The points of curve c in registers.
+template <int D, int DIM>
+__device__ __forceinline__ void load_curve(const CurveArgs& a, int64_t c, float (&b)[D + 1][DIM])
+{
+    const int64_t at = c * ((D + 1) * DIM);
+    if (a.dtype == 0) {
+#pragma unroll
+        for (int m = 0; m <= D; ++m)
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) b[m][k] = __ldg(static_cast<const float*>(a.ctrl) + at + m * DIM + k);
+    } else {
+#pragma unroll
+        for (int m = 0; m <= D; ++m)
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) b[m][k] = load_elem(a.ctrl, a.dtype, at + m * DIM + k);
+    }
+}
+
 constexpr int kFewThreads = 128;
 
 // Points of a small call, one thread per sample or few: the curve's points come
@@ -292,18 +310,7 @@ __global__ void __launch_bounds__(kFewThreads) k_points_few(const CurveArgs a, i
     float t = 0.f, b[D + 1][DIM], P[DIM];
     const float* tc = a.t + c * a.t_stride;
     if (tm == TM_ARRAY) t = __ldg(tc + j);
-    const int64_t at = (int64_t)c * ((D + 1) * DIM);
-    if (a.dtype == 0) {
-#pragma unroll
-        for (int m = 0; m <= D; ++m)
-#pragma unroll
-            for (int k = 0; k < DIM; ++k) b[m][k] = __ldg(static_cast<const float*>(a.ctrl) + at + m * DIM + k);
-    } else {
-#pragma unroll
-        for (int m = 0; m <= D; ++m)
-#pragma unroll
-            for (int k = 0; k < DIM; ++k) b[m][k] = load_elem(a.ctrl, a.dtype, at + m * DIM + k);
-    }
+    load_curve<D, DIM>(a, c, b);
     Eval<VAR, D, DIM> e;
     register_setup<VAR, D, DIM>(b, e);
     const uint32_t key = curve_key<TM_HASH>(a, c);
@@ -329,7 +336,7 @@ __global__ void __launch_bounds__(kFewThreads) k_points_few(const CurveArgs a, i
 // halves with one instruction of two cycles: as many operations per cycle as the
 // scalar forms, for half of the issue slots, and the fused draw-and-measure loop
 // is bound by instruction issue: 28 -> 21.5 lane instructions per point of a 3D
-// cubic.  1,048,576 cubics x 1024 draws: 868 -> 823 us (the FMA pipe that also
+// cubic.  1,048,576 cubics x 1024 draws: 868 -> 799 us (the FMA pipe that also
 // takes the integer multiplies then 76 % busy, issue 70 %; scalar subtractions,
 // additions or square-root sums, 2 or 4 samples side by side and 80 registers
 // all measured slower or the same); 65,536 x 400 of degree 5 68 -> 38 us, 2D
@@ -407,29 +414,64 @@ __device__ __forceinline__ void packed_draws(uint32_t key, uint32_t ja, uint32_t
                     pack2(-1.5f, -1.5f));
 }
 
-// Length over one lane's samples [s, e): the half runs [s, m) and [m, e) side by
+// The order of a length's sum depends on n_t (and on whether the parameters are an
+// array) alone, so that a curve's length to the last bit does not depend on the
+// other curves of the call: a curve's samples are cut into 2^lg runs, a run is
+// summed over its groups of 4 segments in order, and the runs pairwise.  A lane
+// takes a run.  In a call of few curves (FEW) 2^lk lanes share a run's groups, put
+// the group sums into shared memory, and the last of them adds these in order.
+
+constexpr uint32_t kSharedRunSamples = 4096;  // most samples of a curve whose runs are shared
+
+// the groups [g0, g1) of lane `sub` of a run of `groups`
+__device__ __forceinline__ void shared_groups(uint32_t groups, int sub, int lk, uint32_t& g0, uint32_t& g1)
+{
+    const uint32_t each = (groups + (1u << lk) - 1) >> lk;
+    g0 = min(each * sub, groups);
+    g1 = min(g0 + each, groups);
+}
+
+// u = t - 1/2 at the draws of samples ja and jb
+__device__ __forceinline__ f32x2 packed_draw(uint32_t key, uint32_t ja, uint32_t jb)
+{
+    return add2(pack2(hash_one_plus(lowbias32_premixed(key, ja)), hash_one_plus(lowbias32_premixed(key, jb))),
+                pack2(-1.5f, -1.5f));
+}
+
+// Length over a run's samples [s, end): the half runs [s, m) and [m, end) side by
 // side in the halves of the packed registers, their ends joined.  s and m are
 // multiples of 4 and the halves' groups of 4 differ by at most one, so at most
 // 7 samples of the first and 3 of the second half are left for scalar steps.
-// `first`, `last`: the run's end points.
-template <int D, int DIM>
+// `first`, `last`: the run's end points; FEW: these and the length come back in
+// the last of the run's lanes (`sub` of 2^lk), `sums` holds the run's group sums.
+template <int D, int DIM, bool FEW>
 __device__ __forceinline__ float packed_run(const Eval<VAR_HORNER_CENTRED, D, DIM>& e, const TileParams& tp,
-                                            uint32_t s, uint32_t m, uint32_t end, float (&first)[DIM],
-                                            float (&last)[DIM])
+                                            uint32_t s, uint32_t m, uint32_t end, f32x2* sums, int sub, int lk,
+                                            float (&first)[DIM], float (&last)[DIM])
 {
     PackedHorner<D, DIM> h;
     h.setup(e);
     const uint32_t both = min(m - s, end - m) & ~3u;
+    const bool shared = FEW && lk > 0;
+    uint32_t i0 = 0, i1 = both;
+    if (shared) {
+        shared_groups(both / 4, sub, lk, i0, i1);
+        i0 *= 4;
+        i1 *= 4;
+    }
     f32x2 acc2 = 0ull, prev[DIM];
     float acc = 0.f, fb[DIM], pa[DIM], pb[DIM];
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) fb[k] = pa[k] = pb[k] = 0.f;
     if (both > 0) {
         f32x2 u[4];
-        packed_draws(tp.key, s, m, u);
-        h.eval(u[0], prev);  // the run's first segment ends where it starts: length 0
+        packed_draws(tp.key, s + i0, m + i0, u);
+        // the run's first segment ends where it starts: length 0
+        h.eval(FEW && i0 > 0 ? packed_draw(tp.key, s + i0 - 1, m + i0 - 1) : u[0], prev);
 #pragma unroll
         for (int k = 0; k < DIM; ++k) unpack2(prev[k], first[k], fb[k]);
-        for (uint32_t i = 0; i < both; i += 4) {
-            if (i > 0) packed_draws(tp.key, s + i, m + i, u);
+        for (uint32_t i = i0; i < i1; i += 4) {
+            if (i > i0) packed_draws(tp.key, s + i, m + i, u);
             f32x2 gs = 0ull;  // a group's 4 segments are summed first
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
@@ -446,10 +488,24 @@ __device__ __forceinline__ float packed_run(const Eval<VAR_HORNER_CENTRED, D, DI
                 const f32x2 sl = pack2(sqrt_approx(qa), sqrt_approx(qb));
                 gs = g == 0 ? sl : add2(gs, sl);
             }
-            acc2 = add2(acc2, gs);
+            if (shared) sums[i / 4] = gs;
+            else acc2 = add2(acc2, gs);
         }
 #pragma unroll
         for (int k = 0; k < DIM; ++k) unpack2(prev[k], pa[k], pb[k]);
+    }
+    if (shared) {
+        const int base = (threadIdx.x & 31) - sub;
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) {
+            first[k] = __shfl_sync(kFull, first[k], base);
+            fb[k] = __shfl_sync(kFull, fb[k], base);
+        }
+        __syncwarp();
+        if (sub != (1 << lk) - 1) return 0.f;
+        for (uint32_t g = 0; g < both / 4; ++g) acc2 = add2(acc2, sums[g]);
+    }
+    if (both > 0) {
         float aa, ab;
         unpack2(acc2, aa, ab);
         acc = aa + ab;
@@ -483,30 +539,95 @@ __device__ __forceinline__ float packed_run(const Eval<VAR_HORNER_CENTRED, D, DI
     return acc;
 }
 
-// resident blocks per SM that k_length's registers are sized for (the packed
-// form holds its coefficients twice)
-__host__ __device__ constexpr int length_blocks(bool packed, int D, int DIM)
+// Samples of a run of the scalar form, 2^lg runs a curve.  An odd count where the
+// lanes read arrays: with a multiple of 32 they would all read the same bank of the
+// L1 (65,536 x 256 with their own t: 63 us, 24 with 33; x 1024 at shared t 233 and 79).
+__host__ __device__ __forceinline__ uint32_t length_run(uint32_t n_t, int lg, int tm)
 {
-    const int per = (D + 1) * DIM;
-    return packed ? (per <= 6 ? 5 : per <= 12 ? 4 : per <= 16 ? 3 : 2) : per > 20 ? 3 : 4;
+    const uint32_t run = (n_t + (1u << lg) - 1) >> lg;
+    return tm == TM_ARRAY ? run | 1u : run;
 }
 
-// Polyline lengths, 2^lg lanes a curve (65,536 cubics x 400 samples: shared t
-// 36 us, uniform 35, own t 43, against 42, 48 and 52 with a warp per curve): each
-// lane walks a contiguous run of samples (PACKED: centred Horner at pre-mixed
-// draws, two half runs at a time), the segments joining two runs are closed with one shuffle, and the
-// run sums are added over the curve's lanes.
-template <int VAR, int D, int DIM, bool PACKED>
-__global__ void __launch_bounds__(kWarps * 32, (D + 1) * DIM > 20 ? 3 : (D + 1) * DIM > 12 ? 4 : 4)
-    k_length(const CurveArgs a, int tm, int lg)
+// The same over samples [s, end) at any parameters, one sample after the other.
+template <int VAR, int D, int DIM, bool FEW>
+__device__ __forceinline__ float scalar_run(const Eval<VAR, D, DIM>& e, const TileParams& tp, int tm, uint32_t s,
+                                            uint32_t end, float* sums, int sub, int lk, float (&first)[DIM],
+                                            float (&prev)[DIM])
+{
+    const uint32_t groups = s < end ? (end - s - 1) / 4 : 0;  // of 4 segments; up to 3 segments are left
+    const bool shared = FEW && lk > 0;
+    uint32_t g0 = 0, g1 = groups;
+    if (shared) shared_groups(groups, sub, lk, g0, g1);
+    float acc = 0.f;
+    if (s < end) {
+        float t[1];
+        tp.get<1, true>(tm, s + 4 * g0, 1, end, t);
+        e.eval(t[0], first);
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) prev[k] = first[k];
+    }
+    uint32_t j = s + 1 + 4 * g0;
+    for (uint32_t g = g0; g < g1; ++g, j += 4) {
+        // the group's 4 segments are summed first and then added to the run
+        float t[4], gs = 0.f;
+        tp.get<4, true>(tm, j, 1, end, t);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            float P[DIM];
+            e.eval(t[m], P);
+            gs += seg_len<DIM>(P, prev);
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) prev[k] = P[k];
+        }
+        if (shared) sums[g] = gs;
+        else acc += gs;
+    }
+    if (shared) {
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) first[k] = __shfl_sync(kFull, first[k], (threadIdx.x & 31) - sub);
+        __syncwarp();
+        if (sub != (1 << lk) - 1) return 0.f;
+        for (uint32_t g = 0; g < groups; ++g) acc += sums[g];
+    }
+    if (j < end) {
+        float t[4];
+        tp.get(tm, j, 1, end, t);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            if (j + m < end) {
+                float P[DIM];
+                e.eval(t[m], P);
+                acc += seg_len<DIM>(P, prev);
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) prev[k] = P[k];
+            }
+        }
+    }
+    return acc;
+}
+
+// Polyline lengths, 2^lg runs a curve, one lane each (65,536 cubics x 400
+// samples: shared t 33 us, uniform 35, own t 38, against 42, 48 and 52 with a warp
+// per curve): each lane walks a contiguous run of samples (PACKED: centred Horner at
+// pre-mixed draws, two half runs at a time), the segments joining two runs are closed
+// with one shuffle, and the run sums are added over the curve's lanes.  FEW: 2^lk lanes
+// share a run, and where the set-up needs no other lane, every lane loads its curve
+// itself.  A call's time (us, GB300) before and after: 1000 cubics x 256 shared t 4.6 ->
+// 3.1, 1000 quintics x 1024 draws 13.8 -> 4.7, 100 cubics x 65,536 draws 541 -> 70.
+template <int VAR, int D, int DIM, bool PACKED, bool FEW>
+__global__ void __launch_bounds__(kWarps * 32, (D + 1) * DIM > 20 ? 3 : 4)
+    k_length(const CurveArgs a, int tm, int lg, int lk)
 {
     using Smem = TileSmem<D, DIM, 8 * (D + 1) * DIM>;
     __shared__ Smem s_tile[kWarps];
+    __shared__ f32x2 s_sums[FEW ? kWarps : 1][FEW ? kSharedRunSamples / 8 : 1];  // group sums of a warp's curves
     const int lane = threadIdx.x & 31;
     Smem& sm = s_tile[threadIdx.x >> 5];
-    const int G = 1 << lg, cpw = 32 >> lg, grp = lane >> lg, li = lane & (G - 1);
+    const int lanes = FEW ? 1 << lk : 1, ll = FEW ? lg + lk : lg;  // lanes of a run, log2 of a curve's
+    const int B = 1 << lg, cpw = 32 >> ll, grp = lane >> ll, li = lane & ((1 << ll) - 1);
+    const int br = FEW ? li >> lk : li, sub = FEW ? li & (lanes - 1) : 0;
     const uint32_t n_t = (uint32_t)a.n_t;  // unsigned: an index may step past 2^31 - 1
-    const uint32_t run = (n_t + G - 1) >> lg;
+    const uint32_t run = length_run(n_t, lg, tm);
     const int64_t n_units = (a.n_curves + cpw - 1) / cpw;
     const int64_t n_warps = (int64_t)gridDim.x * kWarps;
     TileParams tp;
@@ -515,8 +636,14 @@ __global__ void __launch_bounds__(kWarps * 32, (D + 1) * DIM > 20 ? 3 : (D + 1) 
         const int64_t c0 = u * cpw;
         const int nc = (int)min((int64_t)cpw, a.n_curves - c0);
         Eval<VAR, D, DIM> e;
-        tile_setup<VAR>(a, sm, c0, nc, grp, lane, e);
         const bool live = grp < nc;
+        if constexpr (FEW && (VAR != VAR_HORNER_CENTRED || D < kFp64SetupCentred)) {
+            float b[D + 1][DIM];
+            load_curve<D, DIM>(a, c0 + (live ? grp : 0), b);
+            register_setup<VAR, D, DIM>(b, e);
+        } else {
+            tile_setup<VAR>(a, sm, c0, nc, grp, lane, e);
+        }
         tp.curve(a, tm, c0 + (live ? grp : 0));
         float acc = 0.f, first[DIM], prev[DIM];
 #pragma unroll
@@ -524,58 +651,26 @@ __global__ void __launch_bounds__(kWarps * 32, (D + 1) * DIM > 20 ? 3 : (D + 1) 
         uint32_t jb, je;
         if constexpr (PACKED) {
             // two half runs a lane, in whole groups of 4 samples shared out evenly
-            const uint32_t ng = (n_t + 3) / 4, q = ng >> (lg + 1), r = ng & (2 * G - 1);
-            const uint32_t h0 = 2 * li, h1 = h0 + 1, h2 = h0 + 2;
+            const uint32_t ng = (n_t + 3) / 4, q = ng >> (lg + 1), r = ng & (2 * B - 1);
+            const uint32_t h0 = 2 * br, h1 = h0 + 1, h2 = h0 + 2;
             jb = min(n_t, 4 * (h0 * q + min(h0, r)));
             je = live ? min(n_t, 4 * (h2 * q + min(h2, r))) : jb;
             const uint32_t jm = min(je, 4 * (h1 * q + min(h1, r)));
-            if (jb < je) acc = packed_run<D, DIM>(e, tp, jb, jm, je, first, prev);
+            f32x2* sums = FEW ? s_sums[threadIdx.x >> 5] + (grp * B + br) * (q + (r > 0)) : nullptr;
+            if (FEW || jb < je) acc = packed_run<D, DIM, FEW>(e, tp, jb, jm, je, sums, sub, lk, first, prev);
         } else {
-            jb = min(li * run, n_t);
+            jb = min(br * run, n_t);
             je = live ? min(jb + run, n_t) : jb;
-            if (jb < je) {
-                float t1[1];
-                tp.get<1, true>(tm, jb, 1, je, t1);
-                e.eval(t1[0], first);
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) prev[k] = first[k];
-            }
-            uint32_t j = jb + 1;
-            for (; j + 4 <= je; j += 4) {
-                // the group's 4 segments are summed first and then added to the run
-                float t[4], gs = 0.f;
-                tp.get<4, true>(tm, j, 1, je, t);
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    float P[DIM];
-                    e.eval(t[m], P);
-                    gs += seg_len<DIM>(P, prev);
-#pragma unroll
-                    for (int k = 0; k < DIM; ++k) prev[k] = P[k];
-                }
-                acc += gs;
-            }
-            if (j < je) {
-                float t[4];
-                tp.get(tm, j, 1, je, t);
-#pragma unroll
-                for (int m = 0; m < 3; ++m) {
-                    if (j + m < je) {
-                        float P[DIM];
-                        e.eval(t[m], P);
-                        acc += seg_len<DIM>(P, prev);
-#pragma unroll
-                        for (int k = 0; k < DIM; ++k) prev[k] = P[k];
-                    }
-                }
-            }
+            float* sums = FEW ? reinterpret_cast<float*>(s_sums[threadIdx.x >> 5]) + (grp * B + br) * (run / 4) : nullptr;
+            if (FEW || jb < je) acc = scalar_run<VAR, D, DIM, FEW>(e, tp, tm, jb, je, sums, sub, lk, first, prev);
         }
         float pl[DIM];
 #pragma unroll
-        for (int k = 0; k < DIM; ++k) pl[k] = __shfl_up_sync(kFull, prev[k], 1);
-        if (li > 0 && jb < je) acc += seg_len<DIM>(first, pl);
-        for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);  // over the curve's lanes
-        if (li == 0 && live) a.out[c0 + grp] = acc;
+        for (int k = 0; k < DIM; ++k) pl[k] = __shfl_up_sync(kFull, prev[k], lanes);
+        if (br > 0 && jb < je && sub == lanes - 1) acc += seg_len<DIM>(first, pl);
+        for (int o = B >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o * lanes);  // over the curve's runs
+        if (li == lanes - 1 && live) a.out[c0 + grp] = acc;
+        if (FEW) __syncwarp();  // the next unit's group sums come after this one's are read
     }
 }
 
@@ -660,20 +755,36 @@ LaunchResult launch_length(const CurveArgs& a, int tm, cudaStream_t s, const Lau
 {
     constexpr bool PACKED = VAR == VAR_HORNER_CENTRED;  // the packed form serves the pre-mixed draw
     const bool packed = PACKED && tm == TM_HASH16;
-    auto kern = packed ? k_length<VAR, D, DIM, PACKED> : k_length<VAR, D, DIM, false>;
-    // runs of 16 to 32 samples a lane until a curve has a warp.  By n_t alone:
-    // the order of the sum, and so a curve's length to the last bit, does not
-    // depend on the other curves of the call.
-    // In-kernel draws of 64 samples and more take 4 lanes a curve: nothing is
-    // read per sample, and a lane's set-up and joins serve the longest runs.
+    // Runs of 16 to 32 samples until a curve has 32; of in-kernel draws, where nothing
+    // is read per sample and a lane's set-up and joins serve the longest runs, of up
+    // to 256 samples.
     int lg = 2;
-    if (!packed)
-        while (lg < 5 && a.n_t > (32 << lg)) ++lg;
-    const int64_t units = (a.n_curves + (32 >> lg) - 1) / (32 >> lg);
+    const uint32_t n_t = (uint32_t)a.n_t;
+    while (lg < 5 && n_t > ((packed ? 256u : 32u) << lg)) ++lg;
+    // Lanes that share a run, while their warps fit the SMs at once and (two lanes,
+    // whose second start and joins cost the most) leave the SMs short of warps.  us on
+    // GB300, a lane / 2^lk lanes a run; draws, cubics 32 x 1024 7.7 / 3.8 and 4000 x 1024
+    // 11.2 / 7.9 (8 lanes), 8000 x 1024 11.4 / 13.5 (2); quintics 1000 x 256 5.8 / 3.3,
+    // 1000 x 1024 13.0 / 4.7, 4000 x 4096 21.3 / 28.0 (2); shared t, cubics 1000 x 128
+    // 4.4 / 2.8, 4000 x 256 4.9 / 4.3 (2), 8000 x 256 5.5 / 5.8; Seiler on a grid 1000 x
+    // 256 3.8 / 3.1, 4000 x 256 3.9 / 4.2 (2).
+    const uint32_t groups = packed ? (n_t + 4) >> (lg + 3) : (length_run(n_t, lg, tm) - 1) / 4;
+    auto warps = [&](int k) { return (a.n_curves << (lg + k)) >> 5; };
+    int lk = 0;
+    if (n_t <= kSharedRunSamples)
+        while (lk < 5 - lg && groups >> (lk + 1) >= 1 && warps(lk + 1) <= (int64_t)h.sm_count * 18) ++lk;
+    if (lk == 1 && tm != TM_ARRAY && warps(1) > (int64_t)h.sm_count * 7) lk = 0;
+    // (up to 64 samples, lanes that load their curve themselves are faster throughout:
+    // 65,536 cubics x 64 draws 8.3 -> 7.8)
+    const bool few = lk > 0 || (n_t <= 64 && (VAR != VAR_HORNER_CENTRED || D < kFp64SetupCentred));
+    auto kern = packed ? (few ? k_length<VAR, D, DIM, PACKED, true> : k_length<VAR, D, DIM, PACKED, false>)
+                       : (few ? k_length<VAR, D, DIM, false, true> : k_length<VAR, D, DIM, false, false>);
+    const int cpw = 32 >> (few ? lg + lk : lg);
+    const int64_t units = (a.n_curves + cpw - 1) / cpw;
     const int grid = tile_grid((const void*)kern, units, h.sm_count);
     h.count(h.self);
     h.begin(h.self, s);
-    kern<<<grid, kWarps * 32, 0, s>>>(a, tm, lg);
+    kern<<<grid, kWarps * 32, 0, s>>>(a, tm, lg, lk);
     const cudaError_t err = cudaGetLastError();
     h.end(h.self, s);
     return {1, err};
