@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kSurfWarps * 32, 5) k_surface_bicubic3_warp(co
 }
 
 // General grids: any degrees <= 7, dim 1..4, grid <= 256 per axis.  One warp per
-// unit of work, a block of up to kGridRows rows of one u slab of one volume; a
+// unit of work, a block of up to `rows` rows of one u slab of one volume; a
 // surface is a volume of one slab (degree 0, one grid value) whose v and w are
 // its u and v.  The warp forms Y[j][k][l] = sum_i Bu[i] C[i][j][l][k] and
 // Z[b][k][l] = sum_j Bv[b][j] Y[j][k][l] in warp-private shared memory, l padded
@@ -186,6 +186,7 @@ __global__ void __launch_bounds__(kSurfWarps * 32, 5) k_surface_bicubic3_warp(co
 // 364 -> 155.  4 blocks per SM (3 in 4D) measured best of 3 to 5.
 constexpr int kGridRows = 32;
 constexpr int kGridTile = 128;  // points a warp stages between two write-outs
+constexpr int kMinUnit = 32;    // points of a unit that are worth a warp
 
 // shared memory in floats: the tables, then each warp's C, Y, Z and stage
 struct GridLayout {
@@ -206,8 +207,20 @@ __host__ __device__ inline GridLayout grid_layout(const TensorArgs& a)
     return g;
 }
 
+// The units of a launch: `chunks` of `rows` rows (at most kGridRows) a slab,
+// `each` a warp and one more for the first `more` warps.
+struct GridUnits {
+    int rows, chunks;
+    int64_t each, more;
+};
+
+__device__ __forceinline__ int64_t grid_quotient(int64_t a, int b)
+{
+    return a >> 32 ? a / b : (int64_t)((uint32_t)a / (uint32_t)b);  // (a 64-bit division takes 0.1 us)
+}
+
 template <int L4, int DIM>
-__global__ void __launch_bounds__(kSurfWarps * 32, DIM == 4 ? 3 : 4) k_grid(const TensorArgs a, int chunks)
+__global__ void __launch_bounds__(kSurfWarps * 32, DIM == 4 ? 3 : 4) k_grid(const TensorArgs a, const GridUnits un)
 {
     constexpr int LW = 4 * L4;
     extern __shared__ float4 s_grid[];
@@ -215,9 +228,15 @@ __global__ void __launch_bounds__(kSurfWarps * 32, DIM == 4 ? 3 : 4) k_grid(cons
     const GridLayout g = grid_layout(a);
     const int tid = threadIdx.x, lane = tid & 31;
     const int du = a.du, dv = a.dv, dw = a.dw, nu = a.nu, nv = a.nv, nw = a.nw;
-    bernstein_table(sm, nw, dw, tid, kSurfWarps * 32, LW);
-    bernstein_table(sm + g.bv, nv, dv, tid, kSurfWarps * 32);
-    bernstein_table(sm + g.bu, nu, du, tid, kSurfWarps * 32);
+    // the rows of all three tables side by side (a surface's one slab has the value 1)
+    const int table_rows = nw + nv + (du > 0 ? nu : 0);
+    if (du == 0 && tid == 0) sm[g.bu] = 1.f;
+    for (int r = tid; r < table_rows; r += kSurfWarps * 32) {
+        const bool in_w = r < nw, in_v = !in_w && r < nw + nv;
+        const int row = in_w ? r : in_v ? r - nw : r - nw - nv, d = in_w ? dw : in_v ? dv : du;
+        const int stride = in_w ? LW : d + 1;
+        bernstein_row(sm + (in_w ? 0 : in_v ? g.bv : g.bu) + row * stride, in_w ? nw : in_v ? nv : nu, d, row, stride);
+    }
     __syncthreads();
     const float4* bw4 = s_grid;
     float* mine = sm + g.warp + (tid >> 5) * g.per_warp;
@@ -227,15 +246,14 @@ __global__ void __launch_bounds__(kSurfWarps * 32, DIM == 4 ? 3 : 4) k_grid(cons
     const int q32 = 32 / nw, r32 = 32 - q32 * nw;  // 32 points on: q32 rows and r32 columns
     // a warp takes consecutive units, most of them of one volume: its control
     // points load once per volume, Y is formed once per slab
-    const int64_t n_units = a.n * nu * chunks, n_warps = (int64_t)gridDim.x * kSurfWarps;
-    const int64_t w = (int64_t)blockIdx.x * kSurfWarps + (tid >> 5), each = n_units / n_warps;
-    const int64_t more = n_units - each * n_warps;  // warps with one unit more
-    const int64_t u0 = w * each + min(w, more);
-    int64_t left = each + (w < more ? 1 : 0), slab = u0 / chunks, p = slab / nu, loaded = -1, formed = -1;
-    int ch = (int)(u0 - slab * chunks), ai = (int)(slab - p * nu);
+    const int64_t w = (int64_t)blockIdx.x * kSurfWarps + (tid >> 5);
+    const int64_t u0 = w * un.each + min(w, un.more);
+    int64_t left = un.each + (w < un.more ? 1 : 0), slab = grid_quotient(u0, un.chunks), p = grid_quotient(slab, nu);
+    int64_t loaded = -1, formed = -1;
+    int ch = (int)(u0 - slab * un.chunks), ai = (int)(slab - p * nu);
     for (; left > 0; --left) {
-        const int b0 = ch * kGridRows;
-        const int rows = min(kGridRows, nv - b0);
+        const int b0 = ch * un.rows;
+        const int rows = min(un.rows, nv - b0);
         if (p != loaded) {
             if (a.dtype == 0) {
                 const float* src = static_cast<const float*>(a.ctrl) + p * per;
@@ -312,7 +330,7 @@ __global__ void __launch_bounds__(kSurfWarps * 32, DIM == 4 ? 3 : 4) k_grid(cons
             tile_copy(out + (int64_t)t0 * DIM, stage, cnt * DIM, lane, 32);
             __syncwarp();
         }
-        if (++ch == chunks) {
+        if (++ch == un.chunks) {
             ch = 0;
             ++slab;
             if (++ai == nu) {
@@ -375,7 +393,7 @@ LaunchResult launch_tensor_product(const TensorLaunch& t, cudaStream_t s, const 
     size_t smem = 0;
     int threads = kTensorThreads;
     int64_t work = a.n;
-    int chunks = 1;
+    GridUnits un{kGridRows, 1, 0, 0};
     const bool bicubic3 = a.dw < 0 && a.du == 3 && a.dv == 3 && a.dim == 3 && a.nv % 4 == 0 &&
                           ((uintptr_t)a.out & 15) == 0;
     const bool tricubic1 = a.dw == 3 && a.du == 3 && a.dv == 3 && a.dim == 1 && a.nu <= kVolMaxRows &&
@@ -403,8 +421,16 @@ LaunchResult launch_tensor_product(const TensorLaunch& t, cudaStream_t s, const 
         }
         kern = grid_kernel(a.dw > 3 ? 2 : 1, a.dim);
         threads = kSurfWarps * 32;
-        chunks = (a.nv + kGridRows - 1) / kGridRows;
-        work = (a.n * a.nu * chunks + kSurfWarps - 1) / kSurfWarps;
+        // fewer rows a unit while 32 leave the SMs short of warps (us on GB300, block per
+        // patch before k_grid / always 32 rows / now: one biquadratic patch on 16 x 256
+        // 15.3 / 16.6 / 4.7, 64 of 31 x 31 6.6 / 8.9 / 3.9, 256 of 32 x 33 7.8 / 8.5 / 7.0,
+        // 16 of degree 5 x 4, 1D, 31 x 31 5.5 / 9.4 / 4.1)
+        const int64_t target = (int64_t)h.sm_count * 12;
+        un.rows = a.nv < kGridRows ? a.nv : kGridRows;
+        auto units = [&] { return a.n * a.nu * ((a.nv + un.rows - 1) / un.rows); };
+        while (un.rows > 1 && (un.rows + 1) / 2 * a.nw >= kMinUnit && units() < target) un.rows = (un.rows + 1) / 2;
+        un.chunks = (a.nv + un.rows - 1) / un.rows;
+        work = (units() + kSurfWarps - 1) / kSurfWarps;
         smem = (size_t)grid_layout(a).total * sizeof(float);
         if (smem > 48 * 1024) {
             // the most a launch of this kernel takes, so that calls on several
@@ -414,8 +440,13 @@ LaunchResult launch_tensor_product(const TensorLaunch& t, cudaStream_t s, const 
         }
     }
     const int grid = persistent_grid(kern, threads, smem, h.sm_count, work);
+    if (general) {
+        const int64_t units = a.n * a.nu * un.chunks, warps = (int64_t)grid * kSurfWarps;
+        un.each = units / warps;
+        un.more = units % warps;
+    }
     const SurfTexArgs no_tex{};  // the CUDA-core volume kernel reads no texture
-    void* args[] = {(void*)&a, general ? (void*)&chunks : (void*)&no_tex};
+    void* args[] = {(void*)&a, general ? (void*)&un : (void*)&no_tex};
     h.count(h.self);
     h.begin(h.self, s);
     cudaError_t e = cudaLaunchKernel(kern, dim3(grid), dim3(threads), args, smem, s);

@@ -33,29 +33,31 @@ inline int volume_parts(int64_t n, int nu, int sm_count)
     return parts;
 }
 
-// Bernstein table B[a][i] for n grid values and degree d, via de Casteljau
-// on unit vectors (each entry is a product of lerp weights, exact at ends).
-// Rows of `stride` floats (d + 1 where 0), zeros after the d + 1 values.
-__device__ __forceinline__ void bernstein_table(float* B, int n, int d, int tid, int nthreads, int stride = 0)
+// Row `a` of the Bernstein table of n grid values and degree d: the d + 1 values
+// (products of powers, exact at the ends), zeros up to `stride` floats.
+__device__ __forceinline__ void bernstein_row(float* B, int n, int d, int a, int stride)
 {
-    if (stride == 0) stride = d + 1;
-    for (int a = tid; a < n; a += nthreads) {
-        const float t = n > 1 ? __fdiv_rn((float)a, (float)(n - 1)) : 0.f;
-        const float s = 1.0f - t;
-        // B_i^d(t) = C(d,i) s^(d-i) t^i, built from powers
-        float tp[kTensorMaxDeg + 1], sp[kTensorMaxDeg + 1];
-        tp[0] = sp[0] = 1.f;
-        for (int i = 1; i <= d; ++i) {
-            tp[i] = tp[i - 1] * t;
-            sp[i] = sp[i - 1] * s;
-        }
-        float bin = 1.f;
-        for (int i = 0; i <= d; ++i) {
-            B[a * stride + i] = bin * sp[d - i] * tp[i];
-            bin = bin * (float)(d - i) / (float)(i + 1);
-        }
-        for (int i = d + 1; i < stride; ++i) B[a * stride + i] = 0.f;
+    const float t = n > 1 ? __fdiv_rn((float)a, (float)(n - 1)) : 0.f;
+    const float s = 1.0f - t;
+    // B_i^d(t) = C(d,i) s^(d-i) t^i, built from powers
+    float tp[kTensorMaxDeg + 1], sp[kTensorMaxDeg + 1];
+    tp[0] = sp[0] = 1.f;
+    for (int i = 1; i <= d; ++i) {
+        tp[i] = tp[i - 1] * t;
+        sp[i] = sp[i - 1] * s;
     }
+    float bin = 1.f;
+    for (int i = 0; i <= d; ++i) {
+        B[i] = bin * sp[d - i] * tp[i];
+        bin = bin * (float)(d - i) / (float)(i + 1);
+    }
+    for (int i = d + 1; i < stride; ++i) B[i] = 0.f;
+}
+
+// Bernstein table B[a][i] for n grid values and degree d
+__device__ __forceinline__ void bernstein_table(float* B, int n, int d, int tid, int nthreads)
+{
+    for (int a = tid; a < n; a += nthreads) bernstein_row(B + a * (d + 1), n, d, a, d + 1);
 }
 
 // warp-per-patch kernels: warps per block and the largest u grid they hold
