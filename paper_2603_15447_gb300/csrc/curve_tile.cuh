@@ -733,12 +733,11 @@ LaunchResult launch_points(const CurveArgs& a, int tm, cudaStream_t s, const Lau
     while (lg < 5 && ((a.n_curves << lg) >> 5) < target) ++lg;
     int parts = 1, part_len = 0;
     if (lg == 5 && a.n_curves < target) {
-        const int64_t tiles = (a.n_t + kTileSamples - 1) / kTileSamples;
+        const int64_t tiles = ((int64_t)a.n_t + kTileSamples - 1) / kTileSamples;
         const int64_t want = (target + a.n_curves - 1) / a.n_curves;
         const int64_t per = want >= tiles ? 1 : tiles / want;
-        part_len = (int)per * kTileSamples;
-        parts = (a.n_t + part_len - 1) / part_len;
-        if (parts == 1) part_len = 0;
+        parts = (int)((tiles + per - 1) / per);
+        part_len = parts > 1 ? (int)per * kTileSamples : 0;
     }
     const int64_t units = parts > 1 ? a.n_curves * parts : (a.n_curves + (32 >> lg) - 1) / (32 >> lg);
     const int grid = tile_grid((const void*)kern, units, h.sm_count);
