@@ -167,14 +167,21 @@ def _is_cuda(x):
     return x is not None and not isinstance(x, np.ndarray) and x.is_cuda
 
 
+_raw_stream = None
+
+
 def _stream_handle(stream, device):
+    global _raw_stream
     if stream is None:
+        if _raw_stream is not None and type(device) is int:
+            return _raw_stream(device)
         torch = _torch()
-        if type(device) is not int:
-            return torch.cuda.current_stream(device).cuda_stream
-        # the handle alone: current_stream() builds a Stream object around it
-        # (3.5 us of an 18 us call)
-        return torch._C._cuda_getCurrentRawStream(device)
+        handle = torch.cuda.current_stream(device).cuda_stream
+        # from the second call on the handle alone: current_stream() builds a Stream
+        # object around it (3.5 us of an 18 us call).  The first call has initialised
+        # torch's CUDA state; a torch without the name keeps to current_stream().
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return handle
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
