@@ -435,8 +435,8 @@ bez_status bez_mse_grad(bez_ctx ctx, const float* ctrl, const float* weights, in
  * memory.  The paper has no counterpart; this is a deployment variant of
  * bez_eval_bspline / bez_eval_nurbs.
  *
- * Those calls keep the Bezier spans they extract in a scratch buffer that
- * the context grows with cudaMalloc.  Some callers cannot allow that: code
+ * Those calls keep the Bezier spans of splines whose spans do not fit shared
+ * memory in a scratch buffer that the context grows with cudaMalloc.  Some callers cannot allow that: code
  * that must never synchronise the device (cudaMalloc / cudaFree can), hosts
  * whose memory manager owns all device memory, and plugins that may only use
  * the buffers they are given.  This entry point runs the same kernels with
@@ -453,9 +453,9 @@ bez_status bez_mse_grad(bez_ctx ctx, const float* ctrl, const float* weights, in
  *   larger batches are rejected with BEZ_ERR_INVALID_ARG.
  *
  * The first call on a device looks up the array's device address with that
- * device current; make it before any stream capture.  All calls share the
- * array and each overwrites it, so calls that may overlap on the GPU
- * (different streams without ordering between them) race.  Errors are
+ * device current; make it before any stream capture.  All calls that need the
+ * array share and overwrite it, so order calls that may overlap on the GPU
+ * (on different streams): they would race.  Errors are
  * reported through bez_last_error().  Having no context, the call's
  * launches are not counted or timed by bez_get_stats.
  */

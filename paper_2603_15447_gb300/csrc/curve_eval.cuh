@@ -561,7 +561,7 @@ struct DrawEval<Eval<VAR_HORNER_CENTRED, D, DIM0>> {
 // needs four more registers per lane, and measured slower.)  `first` and
 // `last` return the run's end points for the join with the neighbouring
 // lanes.
-template <class E, int DIM, int UNROLL = 2>
+template <class E, int DIM>
 __device__ __forceinline__ float run_length_h16(const E& e, uint32_t km, int jb, int je, float (&first)[DIM],
                                                 float (&last)[DIM])
 {
@@ -581,7 +581,7 @@ __device__ __forceinline__ float run_length_h16(const E& e, uint32_t km, int jb,
         }
     }
     int g = jb + 4;
-#pragma unroll UNROLL
+#pragma unroll 2
     for (; g + 4 <= je; g += 4) {
         // the group's 4 segments are summed first and then added to the run
         // (as many adds, rounding error growing with the run's groups)

@@ -1,21 +1,22 @@
 // noalloc.cu -- B-spline / NURBS evaluation that allocates no memory.
 //
-// bez_eval_bspline and bez_eval_nurbs keep the Bezier spans they extract in
-// a scratch buffer that the context grows with cudaMalloc.  Some callers
-// cannot allow that: code that must not synchronise the device (cudaMalloc
-// and cudaFree can), hosts whose memory manager owns all device memory and
-// forbids other allocations, and plugins that may only use the buffers they
-// are handed.  bez_eval_spline_noalloc runs the same two kernels with the
-// span scratch in a fixed array compiled into the library instead.
+// bez_eval_bspline and bez_eval_nurbs keep the Bezier spans of splines that
+// do not fit the fused kernel in a scratch buffer that the context grows with
+// cudaMalloc.  Some callers cannot allow that: code that must not synchronise
+// the device (cudaMalloc and cudaFree can), hosts whose memory manager owns all
+// device memory and forbids other allocations, and plugins that may only use
+// the buffers they are handed.  bez_eval_spline_noalloc runs the same kernels (the fused one
+// where the splines fit it), with the span scratch of the others in a fixed
+// array compiled into the library instead.
 //
 // The array is a file-scope __device__ symbol, so every GPU that loads the
 // library holds kNoAllocSpanFloats floats (16 MiB) for the life of the
 // process.  Host code cannot use the symbol's name as a device address; the
 // address is looked up with cudaGetSymbolAddress once per device (on that
 // device's first call, with the device current) and cached.  That first call
-// should therefore come before any stream capture.  All calls share the
-// array: calls that can overlap on the GPU (different streams without
-// ordering) race on it.  Nothing in it has to start at zero: the setup
+// should therefore come before any stream capture.  All calls that need it
+// share the array: such calls that can overlap on the GPU (different streams
+// without ordering) race on it.  Nothing in it has to start at zero: the setup
 // kernel writes every span slot the evaluator reads, including empty spans.
 // The call has no context, so its launches are not counted or timed by
 // bez_get_stats.

@@ -87,9 +87,10 @@ __device__ __forceinline__ bool extract_span_f2(const float* ctrl, const float* 
     const int comps = w ? dim + 1 : dim;
     constexpr int STEPS = P > 1 ? P * (P + 1) / 2 - 1 : 1;  // of either pass
     F2 al[STEPS], be[STEPS];
-    // steps of weight 1 (b is already an argument: clamped ends, repeated knots),
-    // which keep their point as the FP64 form does.  a + 1 (b - a) would lose a
-    // point beside one 2^22 times its size.  (Weight 0 returns a as it is.)
+    // steps of weight 1 (b is already an argument: clamped ends, repeated knots)
+    // keep their point as the FP64 form does.  a + 1 (b - a) would lose a
+    // homogeneous or inserted point beside one 2^20 times its size.  (Weight 0
+    // returns a as it is.)
     unsigned kept = 0;
     {
         const float a = s[P], b = s[P + 1];
