@@ -88,10 +88,9 @@ __device__ __forceinline__ bool extract_span_f2(const float* ctrl, const float* 
     constexpr int STEPS = P > 1 ? P * (P + 1) / 2 - 1 : 1;  // of either pass
     F2 al[STEPS], be[STEPS];
     // steps of weight 1 (b is already an argument: clamped ends, repeated knots)
-    // keep their point as the FP64 form does.  a + 1 (b - a) would lose a
-    // homogeneous or inserted point beside one 2^20 times its size.  (Weight 0
-    // returns a as it is.)
-    unsigned kept = 0;
+    // keep their point as the FP64 form does: they carry the weight 2.  a + 1 (b - a)
+    // would lose a homogeneous or inserted point beside one 2^20 times its size.
+    // (Weight 0 returns a as it is.)
     {
         const float a = s[P], b = s[P + 1];
         int k = 0;
@@ -105,7 +104,7 @@ __device__ __forceinline__ bool extract_span_f2(const float* ctrl, const float* 
 #pragma unroll
             for (int i = P; i >= l; --i, ++k) {
                 be[k] = knot_ratio(b, a, s[P + i - l + 1], a);
-                kept |= s[P + i - l + 1] == b ? 1u << k : 0u;
+                if (s[P + i - l + 1] == b) be[k].h = 2.f;
             }
     }
     bool fine = true;
@@ -132,7 +131,7 @@ __device__ __forceinline__ bool extract_span_f2(const float* ctrl, const float* 
 #pragma unroll
             for (int i = P; i >= l; --i, ++k) {
                 const F2 v = lerp2(Q[i - 1], Q[i], be[k]);
-                Q[i] = (kept >> k) & 1u ? Q[i] : v;
+                Q[i] = be[k].h > 1.5f ? Q[i] : v;
             }
 #pragma unroll
         for (int i = 0; i <= P; ++i) {
