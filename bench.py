@@ -65,7 +65,7 @@ T_OPS, LEN_OPS = 9, 8
 # on the full 65,536 x 512 fit step.
 TRAFFIC_PER_CURVE = {"HORNER_CENTRED": 6330624 / 131072}
 # the kernel behind each headline variant's fused length (cubic 3D, hashed t)
-KERNEL_NAME = {"HORNER_CENTRED": "k_length<2, 3, 3, true> (four lanes per curve, two samples per instruction)", "HALF2": "k_curve_h2"}
+KERNEL_NAME = {"HORNER_CENTRED": "k_length<2, 3, 3, true, false> (four lanes per curve, two samples per instruction)", "HALF2": "k_curve_h2"}
 TRAFFIC_SURFACE_65536 = 12652544 + 742988544
 TRAFFIC_FIT_65536x512 = 540096000 + 120747776
 EVAL_OPS = {"HORNER": 9, "HORNER_CENTRED": 9, "HALF2": 5, "BERNSTEIN": 19, "SEILER": 16, "DECASTELJAU": 36,
@@ -1037,6 +1037,31 @@ def run_reference(args, rank):
             "e2e": {"value": v, "unit": "points/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
 
 
+# What the printed line holds; every other table of a run goes to stderr, as one
+# JSON line of its own (a line of 22 kB did not survive being kept as a log's tail).
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "roofline", "e2e", "gpu_launches", "clocks", "cpu_baseline")
+
+
+def _rounded(x):
+    """Floats to 7 significant digits, through dicts and lists."""
+    if isinstance(x, float):
+        return float(f"{x:.7g}")
+    if isinstance(x, dict):
+        return {k: _rounded(v) for k, v in x.items()}
+    return [_rounded(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def short_line(line):
+    """The printed line of a run: LINE_KEYS, and of every other workload its value, error and share of its peak."""
+    short = {k: line[k] for k in LINE_KEYS if k in line}
+    if "configs" in line:
+        short["configs"] = {
+            name: {"value": c["value"], "unit": c["unit"], "max_norm_err": c.get("max_norm_err"),
+                   "frac": c.get("roofline", {}).get("frac")} for name, c in line["configs"].items()}
+    return _rounded(short)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -1101,6 +1126,9 @@ def main():
             import torch.distributed as dist
             dist.destroy_process_group()
     if line is not None:
+        if args.impl != "reference":
+            print(json.dumps(_rounded(line)), file=sys.stderr, flush=True)
+            line = short_line(line)
         print(json.dumps(line), flush=True)
 
 
