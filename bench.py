@@ -674,7 +674,7 @@ def run_plain(args):
     head = res["DECASTELJAU"]
     return _record("plain: 4,096 cubic 3D curves x 256 shared uniform t, points stored", head["points_per_s"],
                    "points/s", steps, args.warmup, head["ms"], 4096 * 256 * 12 + 4096 * 48 + 1024,
-                   head["kernel_ms"], "k_points (points, de Casteljau)", clocks.summary(),
+                   head["kernel_ms"], "k_points_few (points, de Casteljau)", clocks.summary(),
                    {"max_norm_err": head["max_norm_err"], "bar": FP32_BAR,
                     "variants": {v: {k: x for k, x in r.items() if k != "ms"} for v, r in res.items()},
                     "note": "12.6 MB of output fits in L2; the launch is latency-bound, so its HBM fraction is "
