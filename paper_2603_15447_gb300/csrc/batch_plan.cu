@@ -636,11 +636,12 @@ bez_status bez_batch_create(bez_ctx c, const bez_curve_desc* desc, int64_t n_cur
     b->setup_each = bo ? bo->setup_each_launch != 0 : true;
     b->use_graph = bo ? bo->use_graph != 0 : false;
     char key[160];
-    snprintf(key, sizeof(key), "batch-v3:setup%d:n%d:dim%d:mix%lld/%lld/%lld:deg%d:s%d", b->setup_each ? 1 : 0,
+    snprintf(key, sizeof(key), "batch-v3:setup%d:n%d:dim%d:mix%lld/%lld/%lld:deg%d:s%d%s", b->setup_each ? 1 : 0,
              log2_bucket((double)n_curves), dim,
              (long long)(n_curves ? 100 * n_type[0] / n_curves : 0), (long long)(n_curves ? 100 * n_type[1] / n_curves : 0),
              (long long)(n_curves ? 100 * n_type[2] / n_curves : 0), n_curves ? (int)std::lround((double)deg_sum / n_curves) : 0,
-             log2_bucket(n_curves ? (double)total_samples / n_curves : 0.0));
+             log2_bucket(n_curves ? (double)total_samples / n_curves : 0.0),
+             b->class_dim == dim ? "" : ":one");  // (a shape of its own: one generic kernel)
     b->key = key;
     // launch shape: explicit, tuned or default.  The default goes by the batch's
     // samples: short chunks leave a small batch enough items for every warp, long

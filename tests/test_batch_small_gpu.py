@@ -45,3 +45,20 @@ def test_step(n, launches):
         ref = oracle.bezier(b, oracle.grid(n_s[c]))
         assert normalised_error_ctrl(got[off[c]:off[c + 1]].reshape(1, -1, 2), ref, b).max() <= 1e-6
     assert np.isfinite(got).all()
+
+
+def test_tuned_shapes_are_kept_apart(tmp_path, monkeypatch):
+    """A shape tuned for the class kernels is not taken for a plan of one generic kernel, nor the other way round."""
+    torch = need_gpu()
+    import json
+    from paper_2603_15447_gb300 import bez
+    cache = tmp_path / "tune.json"
+    monkeypatch.setenv("BEZ_AUTOTUNE_CACHE", str(cache))
+    n, n_s, dim = 500, 64, 2
+    i = np.arange(n)
+    desc = bez.descriptors(np.zeros(n), np.full(n, 2), np.full(n, 3), np.full(n, n_s), i * 3 * dim, i * 0, i * n_s * dim)
+    ctrl, out = torch.rand(n * 3 * dim, device="cuda"), torch.empty(n * n_s * dim, device="cuda")
+    for chunk in (0, 512):
+        bez.Batch(desc, dim, ctrl, None, out, autotune=True, chunk=chunk)
+    keys = {k for k in json.loads(cache.read_text()) if k.startswith("batch-v3:setup1:n9:dim2")}
+    assert {k.endswith(":one") for k in keys} == {True, False}
